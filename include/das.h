@@ -273,12 +273,12 @@ size_t das_workspace_size_f8(const das_kv_cache_f8 *cache, int num_q_heads, int 
  * (depths below R, e4m3), so Eqs. 2-3 are evaluated on the stored values.
  * key_depth = value_depth = d is the verify attention of depth d (Sec. 3.4).
  * All other arguments, results and limits as das_mature_v_attention.
- * e4m3 operands are widened exactly to bf16 before the products, except for
- * e4m3 keys with bf16 values at head_dim 128 (Mature-V, key_depth < R =
- * value_depth): there the scores are e4m3 products of the stored keys with
- * each query row split exactly into two e4m3 parts under a power of two per
- * row (exact for elements down to about 2^-9 of the row's largest magnitude,
- * fp32 accumulation), and the queries must be finite.
+ * e4m3 values enter the products exactly (widened).  e4m3 keys are widened
+ * exactly too, or scored by 8-bit products of the stored keys with each query row
+ * split into two or three 8-bit parts under a power of two per row (fp32
+ * accumulation; two parts, at head_dim 128 with bf16 values, are exact for elements
+ * down to about 2^-10 of the row's largest magnitude, three to 2^-17).
+ * With e4m3 keys the queries must be finite; a row that is not gives NaN.
  */
 das_status das_mature_v_attention_f8(const das_kv_cache_f8 *cache, int layer, int key_depth,
                                      int value_depth, const int32_t *prefix_len,

@@ -30,19 +30,14 @@ EncodeTiledFn encode_fn() {
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Tensor map over `rank` dims (innermost first): bf16 elements with 128-byte
-// swizzle, or 8-bit (e4m3) elements without swizzle (their tiles are widened
-// by the kernel, which reads them row by row) or, with swizzle8, with 128-byte
-// swizzle (key tiles of 128-byte rows that the e4m3 MMAs read as they land).
+// swizzle, or 8-bit (e4m3) elements without swizzle (value tiles, widened by
+// the kernel, which reads them row by row) or, with swizzle8, swizzled over
+// their rows of 128 or 64 bytes (key tiles that the e4m3 MMAs read as they land).
+// strides: bytes between elements of dims 1, 2, ..
 bool encode_uncached(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims,
-                     const cuuint32_t *box, bool e4m3, bool swizzle8) {
+                     const cuuint64_t *strides, const cuuint32_t *box, bool e4m3, bool swizzle8) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    cuuint64_t strides[4];
-    cuuint64_t s = e4m3 ? 1 : 2;
-    for (int i = 0; i < rank - 1; ++i) {
-        s *= dims[i];
-        strides[i] = s;
-    }
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     // L2 promotion no wider than one contiguous row: the rows of one head are
     // strided by the other heads, so a 256-byte promotion of a 128-byte row
@@ -53,7 +48,10 @@ bool encode_uncached(CUtensorMap *m, void *base, int rank, const cuuint64_t *dim
                                                             : CU_TENSOR_MAP_L2_PROMOTION_L2_64B;
     return fn(m, e4m3 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
               (cuuint32_t)rank, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              e4m3 && !swizzle8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, promo,
+              e4m3 && !swizzle8        ? CU_TENSOR_MAP_SWIZZLE_NONE
+              : e4m3 && dims[0] == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                      : CU_TENSOR_MAP_SWIZZLE_128B,
+              promo,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -67,6 +65,7 @@ struct MapKey {
     int rank;
     bool e4m3, swizzle8;
     cuuint64_t dims[5];
+    cuuint64_t strides[4];
     cuuint32_t box[5];
 };
 struct MapSlot {
@@ -82,12 +81,16 @@ bool same_key(const MapKey &a, const MapKey &b) {
     if (a.base != b.base || a.rank != b.rank || a.e4m3 != b.e4m3 || a.swizzle8 != b.swizzle8)
         return false;
     for (int i = 0; i < a.rank; ++i)
-        if (a.dims[i] != b.dims[i] || a.box[i] != b.box[i]) return false;
+        if (a.dims[i] != b.dims[i] || a.box[i] != b.box[i] ||
+            (i < a.rank - 1 && a.strides[i] != b.strides[i]))
+            return false;
     return true;
 }
 
+// strides null: dims densely packed in order
 bool encode(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims,
-            const cuuint32_t *box_in, bool e4m3, bool swizzle8 = false) {
+            const cuuint32_t *box_in, bool e4m3, bool swizzle8 = false,
+            const cuuint64_t *strides = nullptr) {
     MapKey key = {};
     key.base = base;
     key.rank = rank;
@@ -98,18 +101,23 @@ bool encode(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims,
         key.dims[i] = dims[i];
         key.box[i] = box_in ? box_in[i] : box_default[i];
     }
-    uint64_t h = 1469598103934665603ull;  // FNV-1a over the key's fields
+    cuuint64_t packed = e4m3 ? 1 : 2;
+    for (int i = 0; i < rank - 1; ++i) {
+        packed *= dims[i];
+        key.strides[i] = strides ? strides[i] : packed;
+    }
+    // a hash of the key's fields, a word at a time (a byte at a time took 1.1 us a call)
+    uint64_t h = 1469598103934665603ull;
     auto mix = [&h](uint64_t v) {
-        for (int i = 0; i < 8; ++i) {
-            h ^= (v >> (8 * i)) & 0xffu;
-            h *= 1099511628211ull;
-        }
+        h = (h ^ v) * 0x9e3779b97f4a7c15ull;
+        h ^= h >> 29;
     };
     mix(reinterpret_cast<uintptr_t>(base));
     mix((uint64_t)rank * 4 + (e4m3 ? 1 : 0) + (swizzle8 ? 2 : 0));
     for (int i = 0; i < rank; ++i) {
         mix(key.dims[i]);
         mix(key.box[i]);
+        if (strides && i < rank - 1) mix(key.strides[i]);
     }
     MapSlot &slot = g_maps[h % kMapSlots];
     {
@@ -119,7 +127,7 @@ bool encode(CUtensorMap *m, void *base, int rank, const cuuint64_t *dims,
             return true;
         }
     }
-    if (!encode_uncached(m, base, rank, key.dims, key.box, e4m3, swizzle8)) return false;
+    if (!encode_uncached(m, base, rank, key.dims, key.strides, key.box, e4m3, swizzle8)) return false;
     std::lock_guard<std::mutex> lock(g_map_mu);
     slot.used = true;
     slot.key = key;
@@ -182,20 +190,38 @@ das_status attention_core(const Shape &c, int layer, Operand key, Operand value,
         return DAS_ERR_WORKSPACE;
 
     const int D = c.head_dim;
-    CUtensorMap tk, tv, tkb, tvb, tq;
-    auto operand_map = [&](CUtensorMap *m, const Operand &o, bool swizzle8) {
-        const cuuint64_t dims[5] = {(cuuint64_t)D, (cuuint64_t)c.kv_heads, (cuuint64_t)c.capacity,
-                                    (cuuint64_t)c.batch, (cuuint64_t)o.slabs};
-        // e4m3: one {D, 1, 64} box per tile; bf16: {64, 1, 64} swizzled panels
-        const cuuint32_t box8[5] = {(cuuint32_t)D, 1, 64, 1, 1};
-        return encode(m, o.base, 5, dims, o.e4m3 ? box8 : nullptr, o.e4m3, swizzle8);
+    CUtensorMap tk, tk2 = {}, tv, tkb, tvb, tq;
+    // Prefix tiles of `keys` positions of one head, `panels` 64-element columns of
+    // them.  e4m3: {D, 1, keys, 1, 1} boxes over [slabs][B][capacity][Hkv][D].
+    // bf16: the columns are a dimension of their own, outside the positions, so
+    // that one {64, keys, panels, 1, 1} box lands as the swizzled panels
+    // [panels][keys][64] that the MMAs read (one copy where there were two or four).
+    // (The kernel for short ranges reads bf16 in {64, 1, keys, 1, 1} boxes of the
+    // e4m3 order.)
+    const bool short_ranges = attn_short_ranges(dev, c.batch, c.kv_heads, c.capacity, D,
+                                                G * max_block, key.e4m3, value.e4m3);
+    auto operand_map = [&](CUtensorMap *m, const Operand &o, int keys, int panels, bool swizzle8) {
+        if (o.e4m3 || short_ranges) {
+            const cuuint64_t dims[5] = {(cuuint64_t)D, (cuuint64_t)c.kv_heads,
+                                        (cuuint64_t)c.capacity, (cuuint64_t)c.batch,
+                                        (cuuint64_t)o.slabs};
+            const cuuint32_t box[5] = {(cuuint32_t)(o.e4m3 ? D : 64), 1, (cuuint32_t)keys, 1, 1};
+            return encode(m, o.base, 5, dims, box, o.e4m3, o.e4m3 && swizzle8);
+        }
+        const cuuint64_t row = (cuuint64_t)c.kv_heads * D * 2;
+        const cuuint64_t dims[5] = {64, (cuuint64_t)c.capacity, (cuuint64_t)(D / 64),
+                                    (cuuint64_t)c.kv_heads, (cuuint64_t)c.batch * o.slabs};
+        const cuuint64_t strides[4] = {row, 128, (cuuint64_t)D * 2, row * c.capacity};
+        const cuuint32_t box[5] = {64, (cuuint32_t)keys, (cuuint32_t)panels, 1, 1};
+        return encode(m, o.base, 5, dims, box, false, false, strides);
     };
-    // e4m3 keys with bf16 values at D = 128 are read by the e4m3 MMAs straight
-    // from the 128-byte-swizzled tile (the kernel's query-split path)
-    const bool key_swizzle8 = key.e4m3 && !value.e4m3 && D == 128;
     const cuuint64_t blk_dims[4] = {(cuuint64_t)D, (cuuint64_t)c.kv_heads, (cuuint64_t)max_block,
                                     (cuuint64_t)c.batch};
-    if (!operand_map(&tk, key, key_swizzle8) || !operand_map(&tv, value, false) ||
+    // e4m3 keys: swizzled where the MMAs read them as they land
+    const bool swizzle8 = !short_ranges || (!value.e4m3 && D == 128);
+    if (!operand_map(&tk, key, kTileKeys, 1, swizzle8) ||
+        (!short_ranges && !operand_map(&tk2, key, 2 * kTileKeys, D / 64, swizzle8)) ||
+        !operand_map(&tv, value, kTileKeys, D / 64, false) ||
         !encode_bf16(&tkb, const_cast<void *>(k_blk), 4, blk_dims) ||
         !encode_bf16(&tvb, const_cast<void *>(v_blk), 4, blk_dims))
         return DAS_ERR_CUDA;
@@ -224,12 +250,13 @@ das_status attention_core(const Shape &c, int layer, Operand key, Operand value,
     const double scale = softmax_scale > 0.f ? (double)softmax_scale : 1.0 / sqrt((double)D);
     p.scale_log2 = (float)(scale * 1.4426950408889634);
     p.num_ctas = attn_grid_size(dev);
+    p.short_ranges = short_ranges;
     attn_workspace_layout(workspace, c.batch, c.kv_heads, p.rows_max, D, p.num_ctas, p);
     // every argument is valid from here on: the only work before the launch
     if (clear_status && cudaMemsetAsync(workspace, 0, kWorkspaceHeader,
                                         static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return DAS_ERR_CUDA;
-    const cudaError_t e = attn_launch(p, D, key.e4m3, value.e4m3, tk, tv, tkb, tvb, tq,
+    const cudaError_t e = attn_launch(p, D, key.e4m3, value.e4m3, tk, tk2, tv, tkb, tvb, tq,
                                       static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? DAS_OK : DAS_ERR_CUDA;
 }

@@ -6,718 +6,214 @@
 // tiles plus one block tile; all pairs' tiles form one list of N tiles, and
 // CTA c of a persistent grid of C CTAs (one per SM) takes the c-th of C
 // equal ranges of that list (block tiles weighted for their extra cost, see
-// kBlockWeight), cut into segments at pair boundaries.  A segment that covers
+// kBlockBytes), cut into segments at pair boundaries.  A segment that covers
 // its pair writes the output.  The others write a partial (O / l and the
 // log-sum-exp of their keys) to the workspace, and merge_kernel, launched
 // right after as a programmatic dependent, combines each split pair's
 // partials by log-sum-exp (8, 4 or 2 segments' loads in flight, chosen per
 // launch).
 //
-// One CTA = four softmax warps + one TMA warp + two MMA warps (+ four
-// conversion warps when prefix keys or values are stored as e4m3).
-//   producer (warp 4): TMA loads of 64-key K and V tiles kStages ahead into a
-//     ring of shared-memory stages, and of each segment's query rows (the
-//     pair's G * max_block rows, ordered i * G + g, which is the order of a
-//     {64, G, max_block} box).
-//   P V issuer (warp 5) and S issuer (warp 6), one elected lane each, each
-//   blocking on its own in-order barriers:
-//       S = Q K^T    tcgen05.mma M=64 N=64 K=D   -> S buffer (k % 4) in TMEM
-//                    (e4m3 keys at D = 128: two e4m3 passes over the query
-//                    rows split exactly into hi + lo, see split_q)
-//       O += P V     tcgen05.mma M=64 N=D K=64   -> O in TMEM
-//       l += P 1     tcgen05.mma M=64 N=8 K=64   -> the rounded row sums
-//     S of tile k is issued once its K has landed (or been widened) and the
-//     softmax warps have read S buffer k % 4, so the tensor core runs up to
-//     four tiles ahead of the softmax.  A stage is refilled once the P V that
-//     read it has completed.
-//   softmax warps: an M=64 MMA puts row r in TMEM lane 32 (r / 16) + r % 16, so
-//     warp w owns rows 16w..16w+15 and two threads share a row (one per half
-//     of the 64 keys).  They load the row's scores (and free the S buffer),
-//     mask and scale them (base 2), keep a reference max m that only moves
-//     when a score exceeds it by more than 2^8 (then O and l are rescaled in
-//     TMEM), write P = 2^(s - m) as bf16 into a 128-byte-swizzled [64 rows]
-//     [64 keys] buffer (the K-major A operand of P V) and accumulate the row
-//     sum of the fp32 weights (for the lse).  The sum of the weights as
-//     rounded to bf16 (for the normalisation, so that the output is a convex
-//     combination of the values with exactly the weights the tensor core
-//     used) is the tensor core's, P times a ones column.  At the end of a
-//     segment they read the O rows and that sum from TMEM and write O / l and
-//     the lse (or the partial).
-// Pairs of at most 16 (32) query rows (decode-shaped calls; D = 128, bf16
-// values, keys bf16 or e4m3 with split-query scores) take the
-// replicated-rows variant: the rows are loaded four (two) times, at
-// MMA rows 0, 16, 32 and 48 (0 and 32), and the softmax warps of copy c take
-// only that copy's quarter (half) of every tile's keys, 8 (16) scores a
-// thread instead of 32.  The rest of each copy's P row stays zero, so P V and
-// the row-sum MMA accumulate each copy's own keys; each copy is a softmax of
-// its own (reference max, sums, O rows), and the copies are combined by
-// log-sum-exp through shared memory at a segment end.
+// The products are formed transposed: keys and head dimensions are the rows
+// (M = 128) of the MMAs and the pair's query rows (G * max_block of them, ordered
+// i * G + g as a {64, G, max_block} box lands, rounded up to N = 16, 32 or 64)
+// their columns:
+//     S^T = K Q^T    two 64-key tiles (a step) at a time, K from shared memory
+//     O^T += V^T P^T V as it lies in shared memory (MN-major)
+//     l   += 1 P^T   the sums of P as rounded
+// so that MMAs and softmax shrink with the number of query rows, the MMAs run
+// at the full M = 128 rate, and a softmax thread owns one key: no exchange
+// between threads is needed in a step but one barrier (with rows in the lanes,
+// a 64-key tile cost a softmax warp about 1000 cycles of dependent latency, and
+// its exchanges; D = 64 and e4m3 tiles, 16 KB, could not be consumed faster).
+//
+// One CTA = four softmax warps (eight for N = 64, two groups of 32 columns) +
+// a producer, a P V and an S warp (+ four conversion warps for e4m3).
+//   S warp: loads K, a slot per step, and issues S^T (and, of a segment's first
+//     step, the scores of a few keys the other way round, from which each row's
+//     first reference is taken).  e4m3 keys: two e4m3 passes over the query
+//     rows split exactly into hi + lo, see split_q.
+//   producer warp: loads the query rows and V; the first steps' K too.
+//   P V warp: O^T += V^T P^T and the row sums, once P is in shared memory.
+//   conversion warps: the query split, and e4m3 V widened to f16 tiles.
+//   softmax warps: thread j takes key j's scores of its group's query rows from
+//     tensor memory, subtracts the rows' references (base 2; a reference only
+//     moves when a score exceeds it by 2^60, or 2^15 for f16 P: then O and the
+//     sums are rescaled in tensor memory), and writes P = 2^(s - m) as bf16 (f16
+//     for widened values) into the swizzled, MN-major P buffer.  The sums of the
+//     fp32 weights (for the lse) stay per thread, in tensor memory, and are added
+//     up at a segment's end; the sum of the rounded weights normalises O, so that
+//     the output is a convex combination of the values with exactly the
+//     weights the tensor core used.
+// Measured (us per call, the kernel with query rows in the lanes -> this one,
+// each with its merge): decode B1 H32/32 P4096 T8 16.7 -> 16.1, B16 ragged P
+// 1024-8192 60.2 -> 58.6, B4 P32768 T16 86.4 -> 86.9, ragged D = 64 B8 32.1 -> 26.4,
+// e4m3 keys B4 P16384 46.2 -> 42.0, e4m3 keys and values B8 ragged 58.1 -> 41.0.
+// Bound by DRAM on the long bf16 calls (6.2 TB/s with all fixed costs), by the
+// softmax step (about 2000 cycles) where keys and values are e4m3.
+//
 // The kernel is launched as a programmatic dependent of the previous kernel
 // in the stream: barrier set-up, the tensor-memory allocation, the work plan
 // (from lengths read before the wait, checked again after it) and an L2
 // prefetch of the first tiles overlap the previous kernel's tail; nothing
 // global is written, and nothing read is used unchecked, before
 // griddepcontrol.wait.  Every wait is bounded (2 s); a time-out sets the
-// status word and stops the CTA's waits.  Tensor memory (512 columns) is
-// freed before the CTA exits.
-#include <cuda_bf16.h>
-
+// status word and stops the CTA's waits.  Tensor memory is freed before the CTA
+// exits.
 #include <algorithm>
 #include <atomic>
 
-#include "das_internal.h"
+#include "das_tc.h"
 
 namespace das {
 namespace tc {
 namespace {
 
-constexpr uint32_t kFull = 0xffffffffu;
-constexpr unsigned long long kWaitNs = 2000000000ull;
-constexpr float kLn2 = 0.6931471805599453f;
-constexpr int kSoftWarps = 4;
-constexpr int kProducerWarp = kSoftWarps;     // TMA loads
-constexpr int kMmaWarp = kSoftWarps + 1;      // tcgen05 MMAs of P V
-constexpr int kSWarp = kSoftWarps + 2;        // tcgen05 MMAs of S
-constexpr int kConvWarp0 = kSoftWarps + 3;    // e4m3 -> bf16 widening (e4m3 variants)
-constexpr int kConvWarps = 4;
-constexpr int kRows = 64;            // M of every MMA (query rows per pair)
-constexpr int kSBufs = 4;            // S buffers in tensor memory
-constexpr int kPrefetchTiles = 2;    // prefix tiles pulled into L2 before the dependency wait
-constexpr int kLongRange = 80;       // ranges longer than this prefetch one tile (measured:
-                                     // long / verify 0.45 us faster, decode and batched not)
-constexpr int kTmemCols = 512;       // S buffers [0, 64 kSBufs), O [64 kSBufs, 64 kSBufs + D),
-                                     // then 8 columns whose first is the rounded row sum
-constexpr float kRescaleLog2 = 8.f;  // move the reference max only beyond 2^8
+constexpr int kPBufs = 2;            // P buffers
+// The reference of a row moves only when a score exceeds it by more than
+// 2^kRescale: P and its sums are floating point, so a low reference costs no
+// precision, and moving it costs a CTA about 4 us.  f16 P (widened values) must
+// stay below 2^16, bf16 P and the fp32 sums of P V far below 2^127.
+// A segment's first reference is the maximum over its first keys: where the scores
+// of a row are all alike, or few, its weights should lie at or just below 1 (bf16
+// holds 1 exactly, and its relative error is half as large just below 1 as just
+// above; with the first key's score alone the largest error of a test's output
+// rose from 9.5e-3 to 1.06e-2 of the row's rms).  32 keys for f16 P (fewer moves)
+// and for pairs of up to kRefTiles tiles, else 16 (us, 32 -> 16: the draft, verify,
+// accept and commit step of B2 92.2 -> 91.0, two calls of B4 P32768 173.1 -> 172.9).
+constexpr float kRescaleBf16 = 60.f, kRescaleF16 = 15.f;
+constexpr int kRefKeys = 32, kRefTiles = 9;
+constexpr float kNoRef = 3e38f;      // -reference of a row without a finite score yet
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ unsigned long long globaltimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait; false after 2 s or once another thread of the CTA gave up.
-__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                       int32_t *status) {
-    const unsigned long long t0 = globaltimer();
-    for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 63u) == 0) {
-            if (*abort_flag) return false;
-            if (globaltimer() - t0 > kWaitNs) {
-                *abort_flag = 1;
-                atomicOr(status, kStatusWaitTimeout);
-                return false;
-            }
-        }
-    }
-}
-__device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                     int32_t *status) {
-#pragma unroll 1
-    for (int i = 0; i < 8; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    return wait_slow(bar, parity, abort_flag, status);
-}
-
-// On the abort path only: wait (at most 20 ms, whatever the abort flag says)
-// for a phase whose completion also means that the copies signalling it
-// have landed, so that no bulk copy into shared memory outlives the CTA.
-__device__ __noinline__ void drain_wait(uint32_t bar, uint32_t parity) {
-    const unsigned long long t0 = globaltimer();
-    while (!mbar_try_wait(bar, parity) && globaltimer() - t0 < 20000000ull) {
-    }
-}
-
-__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0,
-                                       int c1, int c2, int c3, int c4, uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        ".L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
-        "r"(c4), "l"(policy)
-        : "memory");
-}
-// L2 prefetch of one box (no shared memory, no barrier).
-__device__ __forceinline__ void tma_prefetch_5d(const CUtensorMap *map, int c0, int c1, int c2,
-                                                int c3, int c4) {
-    asm volatile("cp.async.bulk.prefetch.tensor.5d.L2.global.tile [%0, {%1, %2, %3, %4, %5}];" ::"l"(
-                     reinterpret_cast<uint64_t>(map)),
-                 "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-                 : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap *map, int c0, int c1, int c2,
-                                                int c3) {
-    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(
-                     reinterpret_cast<uint64_t>(map)),
-                 "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-                 : "memory");
-}
-__device__ __forceinline__ void tma_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0,
-                                       int c1, int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
-}
-
-// ---- tcgen05 ----------------------------------------------------------------
-// Shared-memory matrix descriptor: start, leading / stride byte offsets,
-// descriptor version 1, layout 2 = 128-byte swizzle.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)((lbo >> 4) & 0x3FFF) << 16 |
-           (uint64_t)((sbo >> 4) & 0x3FFF) << 32 | (uint64_t)1 << 46 | (uint64_t)2 << 61;
-}
-// Instruction descriptor of kind::f16: bf16 A and B, fp32 D, majors, N, M.
-__host__ __device__ constexpr uint32_t idesc(int M, int N, int a_mn_major, int b_mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn_major << 15) |
-           ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
-                                    uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(id), "r"(accumulate)
-        : "memory");
-}
-// kind::f8f6f4 with e4m3 A and B (format code 0 for both), fp32 D, both K-major.
-__host__ __device__ constexpr uint32_t idesc_e4m3(int M, int N) {
-    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(id), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void fence_before() {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void fence_after() {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// true on exactly one lane of the (converged) warp
-__device__ __forceinline__ bool elect_one() {
-    uint32_t pred;
-    asm volatile(
-        "{\n .reg .pred P;\n .reg .b32 R;\n elect.sync R|P, 0xffffffff;\n"
-        " selp.u32 %0, 1, 0, P;\n}\n"
-        : "=r"(pred));
-    return pred != 0;
-}
-// 32 lanes x 32 consecutive 32-bit columns; thread t gets lane (base + t).
-// The load and its wait form one statement, so no use of the registers can
-// be scheduled before the data is there.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
-// 32 columns of S for the calling thread (16 lanes x 2 halves): thread t < 16
-// of a warp gets TMEM lane t, columns [c, c + 32), thread t + 16 the same lane,
-// [c + 32, c + 64).  With M = 64 a warp's rows sit in its first 16 lanes, so
-// two threads share each row.
-__device__ __forceinline__ void tmem_ld_half32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x32bx2.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-        "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32], "
-        "32;\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
-// (Replicated rows) the calling thread's 8 scores: lane t < 16 of the warp
-// reads TMEM lane t, columns [0, 8) from taddr, lane t + 16 the same lane,
-// columns [8, 16).
-__device__ __forceinline__ void tmem_ld_half8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 8;\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
-}
-// (Replicated rows, two copies) the calling thread's 16 scores: lane t < 16
-// reads TMEM lane t, columns [0, 16) from taddr, lane t + 16 the same lane,
-// columns [16, 32).
-__device__ __forceinline__ void tmem_ld_half16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-        "%13,%14,%15}, [%16], 16;\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-}
-// The O row of the calling thread's half: with M = 64, thread t < 16 of a warp
-// gets TMEM lane t, columns [64 g, 64 g + 32) for g < D / 64, and thread t + 16
-// the same lane, columns [64 g + 32, 64 g + 64).  All loads are issued before
-// the single wait, so the epilogue pays one TMEM round trip.
-template <int D>
-__device__ __forceinline__ void tmem_ld_orow(uint32_t taddr, float (&v)[D / 2]);
-template <>
-__device__ __forceinline__ void tmem_ld_orow<128>(uint32_t taddr, float (&v)[64]) {
-    uint32_t r[64];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15}, [%64], 32;\n"
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,"
-        "%27,%28,%29,%30,%31}, [%65], 32;\n"
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,"
-        "%43,%44,%45,%46,%47}, [%66], 32;\n"
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,"
-        "%59,%60,%61,%62,%63}, [%67], 32;\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]),
-          "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]),
-          "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]),
-          "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]),
-          "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]),
-          "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-        : "r"(taddr), "r"(taddr + 16), "r"(taddr + 64), "r"(taddr + 80)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 64; ++j) v[j] = __uint_as_float(r[j]);
-}
-template <>
-__device__ __forceinline__ void tmem_ld_orow<64>(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15}, [%32], 32;\n"
-        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,"
-        "%27,%28,%29,%30,%31}, [%33], 32;\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31])
-        : "r"(taddr), "r"(taddr + 16)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-        "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(
-            taddr),
-        "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-        "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-        "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-        "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-        "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-        "r"(__float_as_uint(v[15])), "r"(__float_as_uint(v[16])), "r"(__float_as_uint(v[17])),
-        "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])), "r"(__float_as_uint(v[20])),
-        "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])), "r"(__float_as_uint(v[23])),
-        "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])), "r"(__float_as_uint(v[26])),
-        "r"(__float_as_uint(v[27])), "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])),
-        "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-        : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// Packed fp32 arithmetic (two independent IEEE operations per instruction,
-// bit for bit the scalar results) and the three-input maximum.
-__device__ __forceinline__ void fma2(float &d0, float &d1, float a0, float a1, float b0, float b1,
-                                     float c0, float c1) {
-    asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
-        " mov.b64 c, {%6, %7};\n fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}"
-        : "=f"(d0), "=f"(d1)
-        : "f"(a0), "f"(a1), "f"(b0), "f"(b1), "f"(c0), "f"(c1));
-}
-__device__ __forceinline__ void add2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
-    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
-        " add.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}"
-        : "=f"(d0), "=f"(d1)
-        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ void mul2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
-    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
-        " mul.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}"
-        : "=f"(d0), "=f"(d1)
-        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
-// ---- tile list ----------------------------------------------------------------
-__device__ __forceinline__ int clamp_prefix(const AttnParams &p, int b) {
-    int v = p.prefix_len[b];
-    return v < 0 ? 0 : (v > p.capacity ? p.capacity : v);
-}
-__device__ __forceinline__ int clamp_block(const AttnParams &p, int b) {
-    int v = p.block_len[b];
-    return v < 0 ? 0 : (v > p.max_block ? p.max_block : v);
-}
-__device__ __forceinline__ int tiles_of(int P) { return (P + kTileKeys - 1) / kTileKeys + 1; }
-
-struct Walk {
-    int b, h, t, nt, P, T;
-};
-__device__ __forceinline__ void walk_load_seq(const AttnParams &p, Walk &w) {
-    if (w.b < p.B) {
-        w.P = clamp_prefix(p, w.b);
-        w.T = clamp_block(p, w.b);
-        w.nt = tiles_of(w.P);
-    }
-}
-__device__ __forceinline__ void walk_next(const AttnParams &p, Walk &w) {
-    if (++w.t == w.nt) {
-        w.t = 0;
-        if (++w.h == p.Hkv) {
-            w.h = 0;
-            ++w.b;
-            walk_load_seq(p, w);
-        }
-    }
-}
-
-// Extra weight of a pair's block tile when the list is split.  Ending one
-// segment and starting the next (the mostly empty block tile holding a
-// pipeline slot, the wait for the last P V, the partial write, the next
-// queries) costs a CTA two to three tiles' time (a fit of per-CTA loop times
-// on the batched workload: about 1.1 us per block tile plus 0.65 us per
-// segment, against 0.72 us per tile), so a range that holds a block tile
-// takes three tiles fewer while there is at least one CTA per pair; with
-// more pairs than CTAs nearly every range holds one and the weight would
-// only move work around (weights 1-4 and CTA-per-pair thresholds 1 and 4
-// measured on the decode, long, batched and verify workloads; 3 against 2:
-// long 86.9 -> 86.7 us, the others within 0.1 %).
-constexpr int kBlockWeight = 3;
-constexpr int kCtasPerPairForWeight = 1;
-
-// The split of the tile list: tile x of pair q has weighted position
-// x + beta q; CTA c takes the tiles whose weighted position lies in
-// [c W / C, (c+1) W / C).  beta = kBlockWeight if there are at least
-// kCtasPerPairForWeight CTAs per pair and W >= (2 + beta) C (which leaves no
-// CTA empty: weighted positions are at most 1 + beta apart), else 0.
-struct Split {
-    long long N;  // tiles
-    long long W;  // N + beta * pairs
-    int beta;
-};
-
-// The split, given the total tile count.
-__device__ __forceinline__ Split split_from_total(const AttnParams &p, long long total) {
-    const long long pairs = (long long)p.B * p.Hkv;
-    Split sp;
-    sp.N = total;
-    sp.beta = pairs * kCtasPerPairForWeight <= p.num_ctas &&
-                      total + kBlockWeight * pairs >= (long long)(2 + kBlockWeight) * p.num_ctas
-                  ? kBlockWeight
-                  : 0;
-    sp.W = total + sp.beta * pairs;
-    return sp;
-}
-
-// Clamped length read from L2 (not kept in L1, so that a value read before
-// the dependency wait can never be served stale to a later load).
-__device__ __forceinline__ int len_cg(const int32_t *a, int b, int cap) {
-    const int v = __ldcg(a + b);
-    return v < 0 ? 0 : (v > cap ? cap : v);
-}
-
-// Tiles of one pair of sequence b (0 past the batch); at most 2^25, so sums
-// over 32 sequences fit in 32 bits.
-__device__ __forceinline__ int seq_tiles(const AttnParams &p, int b) {
-    return b < p.B ? tiles_of(clamp_prefix(p, b)) : 0;
-}
-
-__device__ Split split_of(const AttnParams &p) {  // whole warp
-    const int lane = threadIdx.x & 31;
-    long long total = 0;
-    for (int b0 = 0; b0 < p.B; b0 += 32)
-        total += (long long)__reduce_add_sync(kFull, (unsigned)seq_tiles(p, b0 + lane)) * p.Hkv;
-    return split_from_total(p, total);
-}
-
-// a / b for 0 <= a, 0 < b: a 32-bit division when both fit (the usual case;
-// a 64-bit division is a long dependent instruction sequence).
-__device__ __forceinline__ long long udiv(long long a, long long b) {
-    if ((((unsigned long long)a | (unsigned long long)b) >> 32) == 0)
-        return (long long)((uint32_t)a / (uint32_t)b);
-    return a / b;
-}
-
-// The CTA whose weighted range holds weighted position q.
-__device__ __forceinline__ int cta_of_w(long long q, const Split &sp, int C) {
-    return (int)udiv((q + 1) * C - 1, sp.W);
-}
-
-// Range [lo, hi) of this CTA and the walk state of its first tile (a whole
-// warp executes this).  One pass over the sequences: a 32-bit inclusive scan
-// of the per-pair tile counts gives, for sequence b of a chunk, both the
-// tiles and the weighted positions before it; the tiles at the weighted
-// positions c W / C and (c+1) W / C are located in the same pass.
-// P0 / T0: the clamped lengths of sequence `lane` (0 past the batch), given
-// by the caller; with B <= 32 they are all the plan reads.
-__device__ bool plan(const AttnParams &p, int P0, int T0, long long &lo, long long &hi, Walk &w) {
-    const int lane = threadIdx.x & 31;
-    const int nt0 = lane < p.B ? tiles_of(P0) : 0;
-    const Split sp =
-        p.B <= 32 ? split_from_total(p, (long long)__reduce_add_sync(kFull, (unsigned)nt0) * p.Hkv)
-                  : split_of(p);
-    const long long lw = udiv((long long)blockIdx.x * sp.W, p.num_ctas);
-    const long long hw = udiv(((long long)blockIdx.x + 1) * sp.W, p.num_ctas);
-    lo = hi = sp.N;
-    bool have_lo = false;
-    long long run_w = 0, run_t = 0;  // weighted positions / tiles before the chunk
-    for (int b0 = 0; b0 < p.B; b0 += 32) {
-        const int nt = b0 == 0 ? nt0 : seq_tiles(p, b0 + lane);
-        int inc = nt;  // inclusive scan over the chunk
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int u = __shfl_up_sync(kFull, inc, d);
-            if (lane >= d) inc += u;
-        }
-        const int nseq = min(32, p.B - b0);
-        // weighted position after this lane's sequence
-        const long long after_w =
-            run_w + ((long long)inc + (long long)sp.beta * min(lane + 1, nseq)) * p.Hkv;
-        // tile x at weighted position q, q inside sequence f of this chunk
-        auto locate = [&](long long q, int f, Walk *wk) {
-            const int ntf = __shfl_sync(kFull, nt, f);
-            const int excl = __shfl_sync(kFull, inc, f) - ntf;
-            const long long seq_w = run_w + ((long long)excl + (long long)sp.beta * f) * p.Hkv;
-            const long long seq_t = run_t + (long long)excl * p.Hkv;
-            const long long off = q - seq_w;
-            int h = (int)udiv(off, ntf + sp.beta);
-            int t = (int)(off - (long long)h * (ntf + sp.beta));
-            if (t >= ntf) {  // inside a block tile's extra weight: the next pair
-                t = 0;
-                ++h;
-            }
-            if (wk) {
-                wk->b = b0 + f;
-                wk->h = h;
-                wk->t = t;
-                if (b0 == 0) {  // lengths already in registers
-                    wk->P = __shfl_sync(kFull, P0, f);
-                    wk->T = __shfl_sync(kFull, T0, f);
-                    wk->nt = tiles_of(wk->P);
-                } else {
-                    walk_load_seq(p, *wk);
-                }
-                if (wk->h == p.Hkv) {
-                    wk->h = 0;
-                    ++wk->b;
-                    walk_load_seq(p, *wk);
-                }
-            }
-            return seq_t + (long long)h * ntf + t;
-        };
-        if (!have_lo) {
-            const unsigned m = __ballot_sync(kFull, after_w > lw);
-            if (m) {
-                lo = locate(lw, __ffs(m) - 1, &w);
-                have_lo = true;
-            }
-        }
-        if (have_lo) {
-            const unsigned m = __ballot_sync(kFull, after_w > hw);
-            if (m) {
-                hi = locate(hw, __ffs(m) - 1, nullptr);
-                break;
-            }
-        }
-        run_w += ((long long)__shfl_sync(kFull, inc, 31) + (long long)sp.beta * nseq) * p.Hkv;
-        run_t += (long long)__shfl_sync(kFull, inc, 31) * p.Hkv;
-    }
-    return lo < hi;
-}
-
-// Shared memory of one CTA.  Keys and values stored as e4m3 (the depths below
-// R in a das_kv_cache_f8) land in the stage as 8-bit tiles [64 keys][D].
-//   kQSplit (keys e4m3, values bf16, D = 128: Mature-V over a das_kv_cache_f8):
-//     the key tile lands 128-byte swizzled and is read by the S MMAs as it is
-//     (kind::f8f6f4).  The conversion warps split each segment's bf16 query
-//     rows exactly into two e4m3 parts, 2^e q = hi + lo with one power of two
-//     e per row (see split_q), and S = (hi + lo) K^T is two e4m3 products
-//     accumulated in fp32, 2^e times the bf16 product.  The pair's block
-//     tile (bf16 keys) has a bf16 key buffer of its own and bf16 MMAs.
-//   otherwise: the conversion warps widen every e4m3 tile into bf16 tiles, in
-//     the 128-byte-swizzled layout the MMAs read, held in a ring of kConvSlots
-//     slots (tile j in slot j % kConvSlots) rather than one per stage: the
-//     smaller stages then fit 6 (or 7) deep instead of 4, which is what keeps
-//     more DRAM requests in flight per SM.  A pair's block tile is bf16: the
-//     conversion warps load its e4m3-stored operands straight into the ring
-//     slot, the producer the others into the stage.
-template <int D, bool KF8, bool VF8, int NC = 1>
+// Shared memory of one CTA.  A step is one or two consecutive 64-key tiles of
+// a pair (two unless the pair or the range ends, or the second would be a
+// block tile of another element type); its keys are the M = 128 rows of the
+// S^T MMA.
+//   K ring: one slot per step, [128 keys][D] (tile h at key rows 64 h).
+//   V ring: one slot per tile, [64 keys][D]; with e4m3 values only prefix
+//     tiles use it, and the conversion warps widen each into a slot of the W
+//     ring, from which the P V MMAs then read every tile.
+//   bf16 tiles are D / 64 panels of 128-byte rows, 128-byte swizzled; e4m3 key
+//   tiles are rows of D bytes, swizzled over the row (128 or 64 bytes), e4m3
+//   value tiles plain rows.
+// Ring depths, measured (us per two calls): V 4 tiles against 5 at D = 128 bf16,
+// B4 P32768 169.9 / 170.5, decode 32.0 / 32.6 (more loads in flight than needed
+// delay the ones needed first); K 3 slots against 2 for N = 16, decode 32.1 /
+// 32.5; S buffers: as many as tensor memory holds, a K slot is free once S is.
+template <int D, bool KF8, bool VF8, int N>
 struct Layout {
-    static constexpr bool REP = NC > 1;  // NC copies of the query rows (1, 2 or 4)
-    static_assert(NC == 1 || NC == 2 || NC == 4, "copies: 1, 2 or 4");
-    // bf16 keys, or e4m3 keys with the split-query scores; bf16 values; D = 128
-    static_assert(!REP || (!VF8 && D == 128), "replicated rows: bf16 values, D = 128");
-    static constexpr bool kQSplit = KF8 && !VF8 && D == 128;
+    static_assert(N == 16 || N == 32 || N == 64, "query columns: 16, 32 or 64");
     static constexpr bool kConv = KF8 || VF8;
-    // (kQSplit: 4 stages of 24 KB measured faster than 5, e4m3 long 82.0 -> 81.5 us)
-    static constexpr int kStages = kQSplit ? 4 : (KF8 && VF8) ? 7 : kConv ? 6 : 4;
-    static constexpr int kConvSlots = 2;
+    static constexpr int kGroups = N == 16 ? 1 : 2;  // softmax groups of four warps
+    static constexpr int kCols = N / kGroups;        // query columns of a group
+    static constexpr int kSoftWarps = 4 * kGroups;
     static constexpr int kThreads = (kSoftWarps + 3 + (kConv ? kConvWarps : 0)) * 32;
     static constexpr int kPanels = D / 64;
-    static constexpr int kTileBytes = kTileKeys * D * 2;  // a bf16 K or V tile
-    static constexpr int kTile8Bytes = kTileKeys * D;     // an e4m3 tile
-    static constexpr int kKBytes = KF8 ? kTile8Bytes : kTileBytes;  // K part of a stage
-    static constexpr int kVBytes = VF8 ? kTile8Bytes : kTileBytes;  // V part of a stage
-    static constexpr int kStageBytes = kKBytes + kVBytes;
-    static constexpr int kConvBytes =
-        kQSplit ? 0 : (KF8 ? kTileBytes : 0) + (VF8 ? kTileBytes : 0);
-    static constexpr int kQBytes = kPanels * kRows * 128;  // one query buffer
-    static constexpr int kQ8Bytes = kRows * 128;           // one e4m3 query part (D = 128)
-    static constexpr int kPBytes = kRows * kTileKeys * 2;  // one P buffer
-    static constexpr int kStagesOff = 0;
-    static constexpr int kConvOff = kStages * kStageBytes;  // the ring of widened tiles, or
-    // (kQSplit) the block tile's bf16 keys, then hi / lo of both query buffers
-    static constexpr int kBlkKOff = kConvOff;
-    static constexpr int kQ8Off = kConvOff + kTileBytes;
-    static constexpr int kExtraBytes =
-        kQSplit ? kTileBytes + 4 * kQ8Bytes : kConvSlots * kConvBytes;
-    static constexpr int kQOff = kConvOff + kExtraBytes;
-    static constexpr int kPOff = kQOff + 2 * kQBytes;
-    // the B operand of the row-sum MMA: [8][64] bf16, row 0 ones, 128-byte swizzled
-    static constexpr int kOnesOff = kPOff + 2 * kPBytes;
-    static constexpr int kBarOff = kOnesOff + 1024;
-    // barriers: full[kStages], empty[kStages], qfull[2], qempty[2],
-    // sready[kSBufs], sfree[kSBufs], pready[2], pvdone[2], drain[2],
-    // cready[kConvSlots], kfree[kConvSlots], vfree[kConvSlots], qsplit[2], bkfree
-    static constexpr int kNumBars = 2 * kStages + 10 + 2 * kSBufs + 3 * kConvSlots + 3;
-    static constexpr int kMiscOff = kBarOff + kNumBars * 8;
+    static constexpr int kTileBytes = kTileKeys * D * 2;                // a bf16 K or V tile
+    static constexpr int kKBytes = 2 * kTileKeys * D * (KF8 ? 1 : 2);   // a K slot
+    static constexpr int kVBytes = kTileKeys * D * (VF8 ? 1 : 2);       // a V slot
+    static constexpr int kKSlots = KF8 || N == 16 ? 3 : D == 64 ? 4 : 2;
+    static constexpr int kVSlots = VF8 ? 4 : D == 64 ? 8 : 4;
+    static constexpr int kWSlots = VF8 ? (D == 64 ? 4 : 3) : 0;
+    static constexpr int kSBufs = KF8 && D == 128 && N == 64 ? 2 : 3;  // S buffers in tensor memory
+    static constexpr int kQBytes = N * D * 2;    // one bf16 query buffer
+    static constexpr int kQ8Bytes = N * D;       // one 8-bit query part
+    // (e4m3 keys) parts of the query split: the third where widening the keys,
+    // which is exact, was the alternative measured (split_q)
+    static constexpr int kParts = VF8 || D == 64 ? 3 : 2;
+    static constexpr int kPBytes = 2 * kTileKeys * N * 2;
+    static constexpr int kVOff = kKSlots * kKBytes;
+    static constexpr int kWOff = kVOff + kVSlots * kVBytes;
+    static constexpr int kQOff = kWOff + kWSlots * kTileBytes;
+    static constexpr int kQ8Off = kQOff + 2 * kQBytes;  // hi, lo (, lo2)
+    static constexpr int kPOff = kQ8Off + (KF8 ? kParts * kQ8Bytes : 0);
+    // (D = 64) 16 keys x 64 ones (bf16, then f16): the second half of the P V A operand
+    static constexpr int kOnesOff = kPOff + kPBufs * kPBytes;
+    static constexpr int kBarOff = kOnesOff + (D == 128 ? 0 : VF8 ? 4096 : 2048);
+    // barriers: kfull / kempty[kKSlots], vfull / vempty[kVSlots], wready /
+    // wfree[kWSlots], qfull[2], qempty[2], qsplit[2], sready / sfree[kSBufs],
+    // pready[2], pvdone[2], drain[2], rready
+    static constexpr int kNumBars = 2 * (kKSlots + kVSlots + kWSlots) + 13 + 2 * kSBufs;
+    static constexpr int kMiscOff = kBarOff + (kNumBars + 1) / 2 * 16;  // tensor memory base, abort flag
     static constexpr int kLenOff = kMiscOff + 16;  // lengths read before the dependency wait
-    static constexpr int kQeOff = kLenOff + 64 * 4;  // (kQSplit) e of each row, per query buffer
-    // (REP) the segment end's exchange, then (m, l, rounded l) of every MMA
-    // row [kRows][4]; rows are padded by 16 bytes so that consecutive rows
-    // start in different bank groups.  Compacted (e4m3 keys, whose stages
-    // leave too little shared memory for whole rows): a softmax thread holds
-    // D / 2 values of its copy's O row, in NC groups of D / 2 / NC; each
-    // group is combined by the thread of the copy with its index, so a thread
-    // stores only the NC - 1 groups other copies combine: [2 halves][kRows]
-    // [kXchStride] floats.
-    // With bf16 keys there is room for the whole rows: every copy's O row
-    // [kRows][kXchStride] (measured faster for bf16: decode 17.43 -> 17.12 us).
-    static constexpr bool kCompactXch = KF8;
-    static constexpr int kXchStride =
-        !REP ? 0 : kCompactXch ? (NC - 1) * (D / 2 / NC) + 4 : D + 4;
-    static constexpr int kXchOff = (kQeOff + (kQSplit ? 2 * kRows * 4 : 0) + 15) & ~15;
-    static constexpr int kXchBytes =
-        !REP ? 0
-             : ((kCompactXch ? 2 * kRows * kXchStride : kRows * kXchStride) + kRows * 4) * 4;
-    static constexpr int kBytes = kXchOff + kXchBytes + 1024;  // + alignment slack
-    static_assert(kStageBytes % 1024 == 0 && kKBytes % 1024 == 0 && kConvBytes % 1024 == 0,
+    static constexpr int kNmOff = kLenOff + 64 * 4;       // -reference of each query row
+    static constexpr int kAlphaOff = kNmOff + N * 4;      // rescale factors
+    static constexpr int kRedOff = kAlphaOff + N * 4;     // [4 warps][N]
+    static constexpr int kLrOff = kRedOff + 4 * N * 4;    // rounded row sums
+    static constexpr int kQscOff = kLrOff + N * 4;        // score scale of each row, per buffer
+    static constexpr int kBytes = kQscOff + (KF8 ? 2 * N * 4 : 0) + 1024;  // + alignment slack
+    // tensor memory columns: S buffers, O, row sums (D = 128), then what every
+    // lane needs of each query row -- minus its reference and (e4m3 keys) its
+    // score scale, kept here because shared memory is what the kernel runs out
+    // of -- the lanes' parts of the sums of the fp32 weights (registers: 32 more
+    // would spill), and 8 columns of bf16 ones (and 8 of f16 ones), the A operand whose
+    // products are row sums
+    static constexpr int kOCol = kSBufs * N;
+    static constexpr int kLCol = kOCol + N;
+    static constexpr int kNmCol = kLCol + (D == 128 ? N : 0);
+    static constexpr int kScCol = kNmCol + N;
+    static constexpr int kSumCol = kScCol + (KF8 ? N : 0);
+    static constexpr int kRefCol = kSumCol + N;  // scores of a segment's first keys, rows in lanes
+    static constexpr int kOnesCol = kRefCol + kRefKeys;
+    static constexpr int kTmemCols = N == 16 ? 256 : 512;
+    static_assert(kOnesCol + (VF8 ? 16 : 8) <= kTmemCols, "tensor memory");
+    static_assert(kKBytes % 1024 == 0 && kVBytes % 1024 == 0 && kQ8Bytes % 1024 == 0 &&
+                      kPBytes % 1024 == 0 && kNmOff % 16 == 0,
                   "swizzled tiles need 1024-byte alignment");
     static_assert(kBytes <= 232448, "shared memory per CTA");
 };
 
-// K-major 128B-swizzled address of bf16 element (row, col) of a [64][64] panel
-__device__ __forceinline__ uint32_t p_chunk_addr(uint32_t base, int row, int chunk) {
-    return base + row * 128 + ((chunk ^ (row & 7)) << 4);
+// Segment at walk position w: the pair's tiles of the range, `left` tiles of
+// which remain.
+struct Seg {
+    int tiles;   // tiles of the segment
+    int pairs;   // tiles that go two to a step (all but a block tile of another element type)
+    int steps;
+    int nfull;   // leading steps of two full prefix tiles
+    bool blk;    // the segment ends with the pair's block tile
+};
+template <bool kConv>
+__device__ __forceinline__ Seg segment(const Walk &w, int left) {
+    Seg s;
+    s.tiles = min(w.nt - w.t, left);
+    s.blk = w.t + s.tiles == w.nt;
+    s.pairs = s.tiles - (kConv && s.blk ? 1 : 0);
+    s.steps = ((s.pairs + 1) >> 1) + s.tiles - s.pairs;
+    s.nfull = max(0, min(w.t + s.tiles, w.P >> 6) - w.t) >> 1;
+    return s;
 }
-
-// Two e4m3 codes (the low and high byte of a) -> bf16x2 (low, high half):
-// the hardware conversion to f16x2 (exact: every e4m3 value, NaN included, is
-// an f16 value), each half widened to f32 and the pair rounded to bf16x2
-// (exact again: an e4m3 value has at most 4 significant bits).
-__device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t a) {
-    uint32_t h;
-    asm("{\n .reg .b16 t;\n cvt.u16.u32 t, %1;\n cvt.rn.f16x2.e4m3x2 %0, t;\n}\n"
-        : "=r"(h)
-        : "r"(a));
-    float f0, f1;
-    asm("{\n .reg .b16 l, u;\n mov.b32 {l, u}, %2;\n cvt.f32.f16 %0, l;\n cvt.f32.f16 %1, u;\n}\n"
-        : "=f"(f0), "=f"(f1)
-        : "r"(h));
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(f1), "f"(f0));
-    return r;
+// Tiles of step i.
+__device__ __forceinline__ int step_tiles(const Seg &s, int i) {
+    return 2 * i + 2 <= s.pairs ? 2 : 1;
 }
+__device__ __forceinline__ void walk_segment(const AttnParams &p, Walk &w, const Seg &s) {
+    w.t += s.tiles - 1;
+    walk_next(p, w);
+}
+// Valid keys of tile t of the walk's pair.
+__device__ __forceinline__ int tile_keys(const Walk &w, int t) {
+    return t == w.nt - 1 ? w.T : min(kTileKeys, w.P - t * kTileKeys);
+}
+// Ring position: slot and the parity of the phase being waited for.
+template <int SLOTS>
+struct Ring {
+    int slot = 0;
+    uint32_t parity = 0;
+    __device__ __forceinline__ void next() {
+        if (++slot == SLOTS) {
+            slot = 0;
+            parity ^= 1;
+        }
+    }
+};
 
-// Widen an e4m3 tile [64 keys][D] (row-major, as the 8-bit TMA box lands)
-// into the bf16 tile the MMAs read: D / 64 panels of [64 keys][128 bytes],
-// 16-byte chunk j of key r at (j ^ (r % 8)) * 16 (128-byte swizzle).  The 128
-// conversion threads (ct = 0..127) each take 16-element chunks.
+// Widen an e4m3 value tile [64 keys][D] (row-major, as the 8-bit TMA box
+// lands) into the f16 tile the P V MMAs read: D / 64 panels of [64 keys][128
+// bytes], 16-byte chunk j of key r at (j ^ (r % 8)) * 16 (128-byte swizzle).
+// Every e4m3 value is exactly an f16 value, so one conversion per pair does
+// it (bf16 took four).  Keys from nvalid on (anything, NaN included) become
+// zeros.  The 128 conversion threads (ct = 0..127) each take 16-element chunks.
 template <int D>
-__device__ __forceinline__ void widen_tile(uint32_t src, uint32_t dst, int ct) {
+__device__ __forceinline__ void widen_tile(uint32_t src, uint32_t dst, int nvalid, int ct) {
     constexpr int kChunks = kTileKeys * D / 16;
 #pragma unroll
     for (int i = 0; i < kChunks / (kConvWarps * 32); ++i) {
@@ -729,200 +225,423 @@ __device__ __forceinline__ void widen_tile(uint32_t src, uint32_t dst, int ct) {
         const int jj = c & 3;
         const int pnl = D == 128 ? (c >> 2) & 1 : 0;
         const int key = D == 128 ? ((c >> 4) << 1) + (pnl ^ ((c >> 3) & 1)) : c >> 2;
-        const int d0 = pnl * 64 + jj * 16;
-        uint32_t w0, w1, w2, w3;
+        uint32_t w[4];
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3)
-                     : "r"(src + key * D + d0));
-        const uint32_t row = dst + (d0 / 64) * 8192 + key * 128;
-        const int j = (d0 % 64) / 8;  // the first of two 16-byte bf16 chunks
-        // bytes 0,1 / 2,3 of each word into the 16-bit halves of a register
-        auto lo = [](uint32_t w) { return w & 0xFFFFu; };
-        auto hi = [](uint32_t w) { return w >> 16; };
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                         row + ((j ^ (key & 7)) << 4)),
-                     "r"(e4m3x2_to_bf16x2(lo(w0))), "r"(e4m3x2_to_bf16x2(hi(w0))),
-                     "r"(e4m3x2_to_bf16x2(lo(w1))), "r"(e4m3x2_to_bf16x2(hi(w1)))
-                     : "memory");
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                         row + (((j + 1) ^ (key & 7)) << 4)),
-                     "r"(e4m3x2_to_bf16x2(lo(w2))), "r"(e4m3x2_to_bf16x2(hi(w2))),
-                     "r"(e4m3x2_to_bf16x2(lo(w3))), "r"(e4m3x2_to_bf16x2(hi(w3)))
-                     : "memory");
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                     : "r"(src + key * D + pnl * 64 + jj * 16));
+        const uint32_t row = dst + pnl * 8192 + key * 128;
+        const bool keep = key < nvalid;
+        uint32_t h[8];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n cvt.rn.f16x2.e4m3x2 %0, l;\n"
+                " cvt.rn.f16x2.e4m3x2 %1, h;\n}\n"
+                : "=r"(h[2 * u]), "=r"(h[2 * u + 1])
+                : "r"(keep ? w[u] : 0u));
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                             row + (((2 * jj + u) ^ (key & 7)) << 4)),
+                         "r"(h[4 * u]), "r"(h[4 * u + 1]), "r"(h[4 * u + 2]), "r"(h[4 * u + 3])
+                         : "memory");
     }
 }
 
-// Exact split of the query rows for e4m3 keys (D = 128).  Row r of the bf16
-// query buffer q (two 128-byte-swizzled panels of [64 rows][64 dims]) becomes
-// two e4m3 rows hi, lo (128-byte swizzled [64 rows][128 dims]) with
-//   2^e q = hi + lo,  e = 7 - floor(log2 max_d |q_d|)  (clamped to +-120),
-// so that the row's largest element scales into [128, 256).  hi is 2^e q
+// Exact split of the query rows for e4m3 keys.  Row r of the bf16 query
+// buffer q (128-byte-swizzled panels of [N rows][64 dims]) becomes two e4m3
+// rows hi, lo ([N rows][D] bytes, swizzled over the row) with
+//   2^e q = hi + lo,  e the largest with 2^e max_d |q_d| <= 448 (e4m3's
+// largest value; e clamped to +-120),
+// so that the row's largest element scales into (224, 448].  hi is 2^e q
 // rounded to e4m3 (4 significant bits) and lo the rounded remainder: a bf16
 // value has 8 significant bits, so the remainder fits e4m3 exactly unless it
 // falls below e4m3's smallest subnormal (2^-9), i.e. for elements below about
-// 2^-9 of the row's largest.  Thread ct of the 128 conversion threads takes
-// row ct / 2, dims [64 (ct % 2), +64); e is written to qexp[row].  A row of
-// zeros gives e = 0; the query must be finite.
-__device__ __forceinline__ void split_q(uint32_t q, uint32_t hi, uint32_t lo, int *qexp, int ct) {
-    const int row = ct >> 1, half = ct & 1;
-    uint32_t w[32];
+// 2^-9 of the row's largest.  With PARTS = 3 what then remains (at most 2^-10) is
+// rounded to e5m2 (3 significant bits, to 2^-16) as a third part, which takes
+// the split's error below that of the fp32 sums (lse of e4m3 keys and values at
+// D = 64, against 64 bits: 8.3e-8 with two parts, 4.1e-8 with keys widened to
+// bf16).  128 / N threads share a row; qsc[row] becomes
+// the scale of the row's scores, scale_log2 2^-e (NaN for a row with an
+// infinity or NaN).
+template <int D, int N, int PARTS>
+__device__ __forceinline__ void split_q(uint32_t q, uint32_t parts, float *qsc, float scale_log2,
+                                        int ct) {
+    constexpr int kTpr = kConvWarps * 32 / N;  // threads per row
+    constexpr int kCh = D / 8 / kTpr;          // 8-element chunks per thread
+    const int row = ct / kTpr, c0 = (ct % kTpr) * kCh;
+    uint32_t w[kCh][4];
+    uint32_t mb = 0;  // largest magnitude, as bits
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
+    for (int i = 0; i < kCh; ++i) {
+        const int c = c0 + i;
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(w[4 * c]), "=r"(w[4 * c + 1]), "=r"(w[4 * c + 2]), "=r"(w[4 * c + 3])
-                     : "r"(q + half * (kRows * 128) + row * 128 + ((c ^ (row & 7)) << 4)));
-    float mx = 0.f;
+                     : "=r"(w[i][0]), "=r"(w[i][1]), "=r"(w[i][2]), "=r"(w[i][3])
+                     : "r"(q + (c >> 3) * (N * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)));
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
-        mx = fmaxf(mx, fmaxf(fabsf(__uint_as_float(w[i] << 16)),
-                             fabsf(__uint_as_float(w[i] & 0xffff0000u))));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        for (int u = 0; u < 4; ++u)
+            mb = max(mb, max((w[i][u] << 16) & 0x7fff0000u, w[i][u] & 0x7fff0000u));
+    }
+#pragma unroll
+    for (int d = 1; d < kTpr; d <<= 1) mb = max(mb, __shfl_xor_sync(kFull, mb, d));
     int e = 0;
-    if (mx > 0.f && mx <= 3.4e38f) {
-        e = 7 - ((int)((__float_as_uint(mx) >> 23) & 0xffu) - 127);
+    if (mb != 0u) {
+        e = ((mb & 0x7fffffu) <= 0x600000u ? 8 : 7) - ((int)(mb >> 23) - 127);
         e = e < -120 ? -120 : (e > 120 ? 120 : e);
     }
     const float sc = __uint_as_float((uint32_t)(127 + e) << 23);
-    // word i holds dims 2i (low half) and 2i + 1 of the thread's 64
-    uint32_t h[16], l[16];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        const float xa = __uint_as_float(w[i] << 16) * sc;
-        const float xb = __uint_as_float(w[i] & 0xffff0000u) * sc;
-        uint32_t h2, f2, l2;
-        asm("{\n .reg .b16 t;\n cvt.rn.satfinite.e4m3x2.f32 t, %1, %2;\n cvt.u32.u16 %0, t;\n}"
-            : "=r"(h2)
-            : "f"(xb), "f"(xa));
-        asm("{\n .reg .b16 t;\n cvt.u16.u32 t, %1;\n cvt.rn.f16x2.e4m3x2 %0, t;\n}"
-            : "=r"(f2)
-            : "r"(h2));
-        float ha, hb;
-        asm("{\n .reg .b16 a, b;\n mov.b32 {a, b}, %2;\n cvt.f32.f16 %0, a;\n cvt.f32.f16 %1, b;\n}"
-            : "=f"(ha), "=f"(hb)
-            : "r"(f2));
-        asm("{\n .reg .b16 t;\n cvt.rn.satfinite.e4m3x2.f32 t, %1, %2;\n cvt.u32.u16 %0, t;\n}"
-            : "=r"(l2)
-            : "f"(xb - hb), "f"(xa - ha));
-        if (i & 1) {
-            h[i >> 1] |= h2 << 16;
-            l[i >> 1] |= l2 << 16;
-        } else {
-            h[i >> 1] = h2;
-            l[i >> 1] = l2;
+    for (int i = 0; i < kCh; ++i) {
+        uint32_t y[PARTS][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float xa = __uint_as_float(w[i][u] << 16) * sc;
+            float xb = __uint_as_float(w[i][u] & 0xffff0000u) * sc;
+#pragma unroll
+            for (int z = 0; z < PARTS; ++z) {  // the next part of what is left
+                uint32_t c2, f2;
+                if (z < 2)
+                    asm("{\n .reg .b16 t;\n cvt.rn.satfinite.e4m3x2.f32 t, %2, %3;\n"
+                        " cvt.u32.u16 %0, t;\n cvt.rn.f16x2.e4m3x2 %1, t;\n}"
+                        : "=r"(c2), "=r"(f2)
+                        : "f"(xb), "f"(xa));
+                else
+                    asm("{\n .reg .b16 t;\n cvt.rn.satfinite.e5m2x2.f32 t, %2, %3;\n"
+                        " cvt.u32.u16 %0, t;\n cvt.rn.f16x2.e5m2x2 %1, t;\n}"
+                        : "=r"(c2), "=r"(f2)
+                        : "f"(xb), "f"(xa));
+                float fa, fb;
+                asm("{\n .reg .b16 a, b;\n mov.b32 {a, b}, %2;\n cvt.f32.f16 %0, a;\n"
+                    " cvt.f32.f16 %1, b;\n}"
+                    : "=f"(fa), "=f"(fb)
+                    : "r"(f2));
+                xa -= fa;
+                xb -= fb;
+                y[z][u >> 1] = (u & 1) ? y[z][u >> 1] | c2 << 16 : c2;
+            }
         }
-    }
-    // 16-byte chunk c of the 128-byte e4m3 row holds dims 16 c .. 16 c + 15:
-    // this thread's are chunks 4 half .. 4 half + 3
+        // 8 bytes at byte 8 c of the row
+        const int c = c0 + i, x = D == 128 ? row & 7 : (row >> 1) & 3;
+        const uint32_t off = row * D + (((c >> 1) ^ x) << 4) + (c & 1) * 8;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const uint32_t off = row * 128 + (((4 * half + m) ^ (row & 7)) << 4);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(hi + off), "r"(h[4 * m]),
-                     "r"(h[4 * m + 1]), "r"(h[4 * m + 2]), "r"(h[4 * m + 3])
-                     : "memory");
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(lo + off), "r"(l[4 * m]),
-                     "r"(l[4 * m + 1]), "r"(l[4 * m + 2]), "r"(l[4 * m + 3])
-                     : "memory");
+        for (int z = 0; z < PARTS; ++z)
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(parts + z * (N * D) + off),
+                         "r"(y[z][0]), "r"(y[z][1])
+                         : "memory");
     }
-    if (half == 0) qexp[row] = e;
+    if (ct % kTpr == 0)
+        qsc[row] = mb >= 0x7f800000u ? __uint_as_float(0x7fc00000u)
+                                     : scale_log2 * __uint_as_float((uint32_t)(127 - e) << 23);
 }
 
-// Registers a thread of the query-split variant may use: 144 x 352 threads
-// leave room for one merge CTA (128 threads x 116) beside the attention CTA,
-// so the merge kernel is resident before the attention grid ends (measured:
-// the e4m3 long call 89.9 -> 89.0 us against 165 registers, no spills).
-template <int D, bool KF8, bool VF8>
-constexpr int kRegCap = Layout<D, KF8, VF8>::kQSplit ? 144 : 255;
+// N consecutive 32-bit columns of the calling thread's tensor-memory lane
+// (taddr holds the warp's first lane); the loads and their wait form one
+// statement, so no use of the registers can be scheduled before the data is
+// there.
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]);
+template <>
+__device__ __forceinline__ void tmem_ld<16>(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "%14,%15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+template <>
+__device__ __forceinline__ void tmem_ld<32>(uint32_t taddr, float (&v)[32]) {
+    tmem_ld32(taddr, v);
+}
+
+// 16 columns of scores, of the rows' -reference and of their scale in one
+// round trip.
+__device__ __forceinline__ void tmem_ld_scores(uint32_t sa, uint32_t ma, uint32_t ca, float *v,
+                                               float (&m)[16], float (&c)[16]) {
+    uint32_t a[16], b[16], d[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "%14,%15}, [%48];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,"
+        "%28,%29,%30,%31}, [%49];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,"
+        "%44,%45,%46,%47}, [%50];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]),
+          "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]),
+          "=r"(a[13]), "=r"(a[14]), "=r"(a[15]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]),
+          "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]),
+          "=r"(b[11]), "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15]), "=r"(d[0]),
+          "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7]),
+          "=r"(d[8]), "=r"(d[9]), "=r"(d[10]), "=r"(d[11]), "=r"(d[12]), "=r"(d[13]),
+          "=r"(d[14]), "=r"(d[15])
+        : "r"(sa), "r"(ma), "r"(ca)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        v[j] = __uint_as_float(a[j]);
+        m[j] = __uint_as_float(b[j]);
+        c[j] = __uint_as_float(d[j]);
+    }
+}
+// N columns from each of two places, in one round trip.
+template <int N>
+__device__ __forceinline__ void tmem_ld_two(uint32_t xa, uint32_t ya, float *x, float (&y)[N]);
+template <>
+__device__ __forceinline__ void tmem_ld_two<16>(uint32_t xa, uint32_t ya, float *x, float (&y)[16]) {
+    uint32_t a[16], b[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "%14,%15}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,"
+        "%28,%29,%30,%31}, [%33];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]),
+          "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]),
+          "=r"(a[13]), "=r"(a[14]), "=r"(a[15]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]),
+          "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]),
+          "=r"(b[11]), "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15])
+        : "r"(xa), "r"(ya)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        x[j] = __uint_as_float(a[j]);
+        y[j] = __uint_as_float(b[j]);
+    }
+}
+
+template <>
+__device__ __forceinline__ void tmem_ld_two<32>(uint32_t xa, uint32_t ya, float *x, float (&y)[32]) {
+    uint32_t a[32], b[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%64];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,"
+        "%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%65];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]),
+          "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]),
+          "=r"(a[13]), "=r"(a[14]), "=r"(a[15]), "=r"(a[16]), "=r"(a[17]), "=r"(a[18]),
+          "=r"(a[19]), "=r"(a[20]), "=r"(a[21]), "=r"(a[22]), "=r"(a[23]), "=r"(a[24]),
+          "=r"(a[25]), "=r"(a[26]), "=r"(a[27]), "=r"(a[28]), "=r"(a[29]), "=r"(a[30]),
+          "=r"(a[31]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]),
+          "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]),
+          "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15]), "=r"(b[16]), "=r"(b[17]),
+          "=r"(b[18]), "=r"(b[19]), "=r"(b[20]), "=r"(b[21]), "=r"(b[22]), "=r"(b[23]),
+          "=r"(b[24]), "=r"(b[25]), "=r"(b[26]), "=r"(b[27]), "=r"(b[28]), "=r"(b[29]),
+          "=r"(b[30]), "=r"(b[31])
+        : "r"(xa), "r"(ya)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        x[j] = __uint_as_float(a[j]);
+        y[j] = __uint_as_float(b[j]);
+    }
+}
+
+// The barrier of softmax group 0 or 1, and whether any of its threads says so.
+template <int ID>
+__device__ __forceinline__ bool bar_any(bool x) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n barrier.cta.red.or.pred p, %2, 128, q;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(r)
+        : "r"((uint32_t)x), "n"(ID)
+        : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ bool soft_any(int group, bool x) {
+    return group == 0 ? bar_any<1>(x) : bar_any<2>(x);
+}
+__device__ __forceinline__ void soft_sync(int group) {
+    if (group == 0)
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+    else
+        asm volatile("bar.sync 2, 128;" ::: "memory");
+}
+
+// The lane's columns from taddr: x, or what they hold plus x.  The stores are
+// waited for by the next call, or by whoever reads them.
+template <int NC>
+__device__ __forceinline__ void tmem_accumulate(uint32_t taddr, float (&x)[NC], bool first) {
+    if (!first) {
+        float o[NC];
+        tmem_wait_st();
+        tmem_ld<NC>(taddr, o);
+#pragma unroll
+        for (int j = 0; j < NC; j += 2) add2(x[j], x[j + 1], x[j], x[j + 1], o[j], o[j + 1]);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; c += 16) {
+        float o[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) o[j] = x[c + j];
+        tmem_st16(taddr + c, o);
+    }
+}
+
+// NC values from shared memory into every lane's columns of tensor memory.
+template <int NC>
+__device__ __forceinline__ void row_values_to_tmem(uint32_t src, uint32_t dst) {
+#pragma unroll
+    for (int c = 0; c < NC; c += 16) {
+        float x[16];
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+            const float4 y = lds4(src + 4 * (c + j));
+            x[j] = y.x;
+            x[j + 1] = y.y;
+            x[j + 2] = y.z;
+            x[j + 3] = y.w;
+        }
+        tmem_st16(dst + c, x);
+    }
+    tmem_wait_st();
+}
+
+// A softmax group's slice of a P buffer: the 2 NC bytes of row `key` that hold
+// its columns.  With two groups the swizzle of P puts them in the row's other
+// half for keys with bit 2 set (128-byte rows at N = 64, 64-byte rows at N = 32).
+template <int N>
+__device__ __forceinline__ uint32_t slice_at(uint32_t pbuf, int group, int key) {
+    return pbuf + key * (2 * N) + (N == 16 ? 0 : (group ^ ((key >> 2) & 1)) * N);
+}
+
+// The maximum (MAX; NaN ignored) or sum of x[r] over the warp's 32 lanes, for
+// each of the NC query rows of its group, into red[r] (shared memory).  The
+// values cross through the warp's rows of the group's slice of a P buffer, half
+// of the rows at a time as fp32: 16 bytes out, 4 bytes in, 16 lanes a thread
+// (31 shuffles or 32 redux instead took 870 and 2900 cycles at NC = 32).
+template <bool MAX, int NC, int N>
+__device__ __forceinline__ void lane_reduce(const float (&x)[NC], uint32_t pbuf, uint32_t red,
+                                            int group, int key) {
+    constexpr int H = NC / 2;  // rows a round: 4 H = 2 NC bytes a lane
+    constexpr int C = H / 4;   // 16-byte chunks a lane
+    const int lane = key & 31, row = lane & (H - 1), k0 = (key & 96) + lane / H * H;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (h) __syncwarp();
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const float *y = x + h * H + 4 * c;
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(
+                             slice_at<N>(pbuf, group, key) + ((c ^ (key & (C - 1))) << 4)),
+                         "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3])
+                         : "memory");
+        }
+        __syncwarp();
+        float y[H];  // all loads first: one latency
+#pragma unroll
+        for (int i = 0; i < H; ++i)
+            y[i] = lds(slice_at<N>(pbuf, group, k0 + i) + (((row >> 2) ^ (i & (C - 1))) << 4) +
+                       (row & 3) * 4);
+#pragma unroll
+        for (int d = H / 2; d > 0; d >>= 1)
+#pragma unroll
+            for (int i = 0; i < d; ++i) y[i] = MAX ? fmaxf(y[i], y[i + d]) : y[i] + y[i + d];
+        float r = y[0];
+#pragma unroll
+        for (int d = H; d < 32; d <<= 1) {
+            const float o = __shfl_xor_sync(kFull, r, d);
+            r = MAX ? fmaxf(r, o) : r + o;
+        }
+        if (lane < H) sts(red + (h * H + row) * 4, r);
+    }
+}
+
+// 1 / x to within an ulp (x > 0; 0 for x = 0)
+__device__ __forceinline__ float inverse(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return x > 0.f ? fmaf(r, fmaf(-x, r, 1.f), r) : 0.f;
+}
+
+// Registers a thread may use, so that a merge CTA (one warp in each of the SM's
+// four register files of 512 x 32) fits beside the attention CTA: 192 with 7
+// warps (two a file) leave 128, 128 with 11 (three a file) too.  bf16 with N = 64
+// would spill at 128 (B16 ragged 241.0 instead of 238.2 us): 144 leave 80, enough
+// for all merge variants but the largest.  15 warps (four a file) leave no
+// room at 128, and fewer would spill.  Where the merge CTA did not fit, a
+// draft, verify, accept and commit step of B2 took 98.7 us instead of 93.8.
+template <int D, bool KF8, bool VF8, int N>
+constexpr int kRegCap = Layout<D, KF8, VF8, N>::kThreads <= 224 ? 192
+                        : Layout<D, KF8, VF8, N>::kConv || N < 64 ? 128
+                                                                  : 144;
 
 // KF8 / VF8: prefix keys / values are e4m3 (tm_k / tm_v are 8-bit maps).
-// NC > 1 (D = 128, bf16 values, at most 64 / NC query rows per pair):
-// replicated rows.  The pair's rows are loaded NC times, copy c at MMA rows [c 64 / NC,
-// (c + 1) 64 / NC), so that the softmax warps of copy c take only keys
-// [c 64 / NC, (c + 1) 64 / NC) of each tile (32 / NC a thread instead of 32).
-// The other keys of their P rows stay zero (the P buffers are cleared once),
-// so P V accumulates each copy's own keys, and each copy keeps its own
-// reference max, sums and O rows; at a segment end the copies are combined
-// by log-sum-exp through shared memory.
-template <int D, bool KF8, bool VF8, int NC>
-__global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
-    __maxnreg__((kRegCap<D, KF8, VF8>)) attn_kernel(const __grid_constant__ CUtensorMap tm_k,
-                   const __grid_constant__ CUtensorMap tm_v,
-                   const __grid_constant__ CUtensorMap tm_kb,
-                   const __grid_constant__ CUtensorMap tm_vb,
-                   const __grid_constant__ CUtensorMap tm_q, const AttnParams p) {
-    using Lt = Layout<D, KF8, VF8, NC>;
-    constexpr bool REP = Lt::REP;
-    constexpr int kStages = Lt::kStages;
+// N: query columns of the MMAs (16, 32 or 64; G * max_block rows rounded up).
+template <int D, bool KF8, bool VF8, int N>
+__global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
+    __maxnreg__((kRegCap<D, KF8, VF8, N>))
+    attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_k2,
+                const __grid_constant__ CUtensorMap tm_v,
+                const __grid_constant__ CUtensorMap tm_kb, const __grid_constant__ CUtensorMap tm_vb,
+                const __grid_constant__ CUtensorMap tm_q, const AttnParams p) {
+    using Lt = Layout<D, KF8, VF8, N>;
+    constexpr bool kConv = Lt::kConv;
+    constexpr int KS = Lt::kKSlots, VS = Lt::kVSlots, WS = VF8 ? Lt::kWSlots : 1;
+    constexpr int kSBufs = Lt::kSBufs, kSoftWarps = Lt::kSoftWarps;
+    constexpr int kProducerWarp = kSoftWarps;   // TMA loads
+    constexpr int kMmaWarp = kSoftWarps + 1;    // MMAs of P V
+    constexpr int kSWarp = kSoftWarps + 2;      // MMAs of S
+    constexpr int kConvWarp0 = kSoftWarps + 3;  // (e4m3) query split, widening
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(sm);
-    const uint32_t bars = sbase + Lt::kBarOff;
-    const uint32_t b_full = bars, b_empty = bars + 8 * kStages, b_qfull = b_empty + 8 * kStages,
-                   b_qempty = b_qfull + 16, b_sready = b_qempty + 16,
-                   b_sfree = b_sready + 8 * kSBufs, b_pready = b_sfree + 8 * kSBufs,
-                   b_pvdone = b_pready + 16, b_drain = b_pvdone + 16,
-                   b_cready = b_drain + 16, b_kfree = b_cready + 8 * Lt::kConvSlots,
-                   b_vfree = b_kfree + 8 * Lt::kConvSlots,
-                   b_qsplit = b_vfree + 8 * Lt::kConvSlots, b_bkfree = b_qsplit + 16;
-    constexpr int kSlots = Lt::kConvSlots;
-    constexpr bool kQSplit = Lt::kQSplit;
-    int *qexp = reinterpret_cast<int *>(sm + Lt::kQeOff);  // [2][kRows]
-    // where the MMAs read tile j's bf16 K and V (stage s = j % kStages): the
-    // TMA tile in the stage, or the ring slot j % kSlots the conversion warps
-    // widened it into
-    const uint32_t kconv0 = sbase + Lt::kConvOff, vconv0 = kconv0 + (KF8 ? Lt::kTileBytes : 0);
-    auto k_src = [&](int st, long long j) {
-        return KF8 ? kconv0 + (int)(j % kSlots) * Lt::kConvBytes : sbase + st * Lt::kStageBytes;
-    };
-    auto v_src = [&](int st, long long j) {
-        return VF8 ? vconv0 + (int)(j % kSlots) * Lt::kConvBytes
-                   : sbase + st * Lt::kStageBytes + Lt::kKBytes;
-    };
+    const uint32_t b_kfull = sbase + Lt::kBarOff, b_kempty = b_kfull + 8 * KS,
+                   b_vfull = b_kempty + 8 * KS, b_vempty = b_vfull + 8 * VS,
+                   b_wready = b_vempty + 8 * VS, b_wfree = b_wready + 8 * Lt::kWSlots,
+                   b_qfull = b_wfree + 8 * Lt::kWSlots, b_qempty = b_qfull + 16,
+                   b_qsplit = b_qempty + 16, b_sready = b_qsplit + 16, b_sfree = b_sready + 8 * Lt::kSBufs,
+                   b_pready = b_sfree + 8 * Lt::kSBufs,
+                   b_pvdone = b_pready + 16, b_drain = b_pvdone + 16, b_rready = b_drain + 16;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sm + Lt::kMiscOff);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + Lt::kMiscOff + 4);
-    // a ring slot is written for tile j once the MMAs of tile j - kSlots that
-    // read it have completed (kfree after S, vfree after P V).  Only the
-    // conversion warps wait on kfree / vfree, and they wait for every tile in
-    // order: a parity wait is exact only when the barrier is at most one phase
-    // behind, which a thread that skipped tiles (the producer, which runs
-    // kStages tiles ahead of P V) could not ensure.
-    auto slot_free = [&](uint32_t bar, long long j) {
-        return j < kSlots || wait(bar + 8 * (int)(j % kSlots),
-                                  (uint32_t)(((j - kSlots) / kSlots) & 1), abort_flag, p.status);
-    };
+    const uint32_t abort_flag = sbase + Lt::kMiscOff + 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
+    // barrier i's wait for a phase of that parity: exact, because every waiter
+    // is at most one phase behind
+    auto await = [&](uint32_t bar, int i, uint32_t parity) {
+        return wait(bar + 8 * i, parity & 1u, abort_flag, p.status);
+    };
 
     // set-up that touches no global memory: it may overlap the previous
     // kernel in the stream (programmatic dependent launch)
     auto init_bars = [&]() {  // one thread
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(b_full + 8 * s, 1);
-            mbar_init(b_empty + 8 * s, 1);
+        for (int s = 0; s < KS; ++s) {
+            mbar_init(b_kfull + 8 * s, 1);
+            mbar_init(b_kempty + 8 * s, 1);
+        }
+        for (int s = 0; s < VS; ++s) {
+            mbar_init(b_vfull + 8 * s, 1);
+            mbar_init(b_vempty + 8 * s, VF8 ? kConvWarps : 1);
+        }
+        for (int s = 0; s < Lt::kWSlots; ++s) {
+            mbar_init(b_wready + 8 * s, kConvWarps);
+            mbar_init(b_wfree + 8 * s, 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(b_qfull + 8 * i, 1);
-            // kQSplit: the last S of the segment and every softmax warp, once
-            // it has read its row's e (the next split overwrites it)
-            mbar_init(b_qempty + 8 * i, kQSplit ? 1 + kSoftWarps : 1);
-            mbar_init(b_pready + 8 * i, kSoftWarps);
+            // e4m3 keys: the segment's last S, and every softmax warp once it
+            // has read the row scales
+            mbar_init(b_qempty + 8 * i, KF8 ? 1 + kSoftWarps : 1);
             mbar_init(b_qsplit + 8 * i, kConvWarps);
+            mbar_init(b_pready + 8 * i, kSoftWarps);
+            mbar_init(b_pvdone + 8 * i, 1);
+            mbar_init(b_drain + 8 * i, 1);
         }
-        mbar_init(b_bkfree, 1);
+        mbar_init(b_rready, 1);
         for (int i = 0; i < kSBufs; ++i) {
             mbar_init(b_sready + 8 * i, 1);
             mbar_init(b_sfree + 8 * i, kSoftWarps);
         }
-        mbar_init(b_pvdone, 1);
-        mbar_init(b_pvdone + 8, 1);
-        mbar_init(b_drain, 1);
-        mbar_init(b_drain + 8, 1);
-        if (Lt::kConv)
-            for (int c = 0; c < kSlots; ++c) {
-                mbar_init(b_cready + 8 * c, kConvWarps);
-                mbar_init(b_kfree + 8 * c, 1);
-                mbar_init(b_vfree + 8 * c, 1);
-            }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     };
     int *len_sm = reinterpret_cast<int *>(sm + Lt::kLenOff);  // [0, 32) P, [32, 64) T
@@ -930,13 +649,13 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
     const bool spec = p.B <= 32;
     if (threadIdx.x == 0) {
         init_bars();
-        *abort_flag = 0;
+        sts(abort_flag, 0.f);
     }
     if (warp == 0) {
         asm volatile(
             "tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                 smem_u32(const_cast<uint32_t *>(tmem_slot))),
-            "n"(kTmemCols));
+            "n"(Lt::kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     // The lengths as they read before the dependency wait (a kernel before
@@ -947,24 +666,20 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
         len_sm[lane0] = lane0 < p.B ? len_cg(p.prefix_len, lane0, p.capacity) : 0;
         len_sm[32 + lane0] = lane0 < p.B ? len_cg(p.block_len, lane0, p.max_block) : 0;
     }
-    if (threadIdx.x < 64) {  // the row-sum MMA's B operand: row 0 of [8][64] bf16 ones
-        const uint32_t one2 = threadIdx.x < 8 ? 0x3F803F80u : 0u;
+    if (D == 64 && threadIdx.x < 128) {  // 2 KB of bf16 ones (and 2 KB of f16 ones)
         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
                          sbase + Lt::kOnesOff + threadIdx.x * 16),
-                     "r"(one2)
+                     "r"(0x3F803F80u)
                      : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    if (REP) {  // both P buffers start (and, outside each copy's keys, stay) zero
-        for (int i = threadIdx.x; i < 2 * Lt::kPBytes / 16; i += Lt::kThreads)
+        if (VF8)
             asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
-                             sbase + Lt::kPOff + i * 16),
-                         "r"(0u)
+                             sbase + Lt::kOnesOff + 2048 + threadIdx.x * 16),
+                         "r"(0x3C003C00u)
                          : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == kProducerWarp && elect_one()) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_k)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_k2)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_v)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_q)) : "memory");
     }
@@ -972,17 +687,23 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (D == 128 && warp < 4) {  // (their readers wait for P, which these warps hand on)
+        const uint32_t at = tmem + ((uint32_t)(warp * 32) << 16) + Lt::kOnesCol;
+        tmem_fill8(at, 0x3F803F80u);
+        if (VF8) tmem_fill8(at + 8, 0x3C003C00u);
+    }
 
     // The plan from the lengths as they read before the dependency wait;
     // after the wait they are read again and the plan is kept only if every
     // length is unchanged.
-    long long lo = 0, hi = 0, ntiles = 0;
+    long long lo = 0, hi = 0;
+    int ntiles = 0;
     Walk w0 = {0, 0, 0, 1, 0, 0};
     int sP = 0, sT = 0;
     if (spec) {
         sP = len_sm[lane0];
         sT = len_sm[32 + lane0];
-        ntiles = plan(p, sP, sT, lo, hi, w0) ? hi - lo : 0;
+        ntiles = plan(p, sP, sT, lo, hi, w0) ? (int)(hi - lo) : 0;
         // While the kernels before this one finish, pull the range's first
         // prefix tiles into L2 (the cache is L2-coherent: if a kernel before
         // this one writes them, the loads after the wait still see its data).
@@ -994,126 +715,157 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
 #pragma unroll
                 for (int dp = 0; dp < Lt::kPanels; ++dp)
                     tma_prefetch_4d(&tm_q, dp * 64, wp.h * p.G, 0, wp.b);
-            const int prefetch = ntiles > kLongRange ? 1 : kPrefetchTiles;
-            for (long long j = 0; j < ntiles && j < prefetch && wp.t < wp.nt - 1; ++j) {
+            const int prefetch = ntiles > kLongRange ? 0 : kPrefetchTiles;
+            for (int j = 0; j < ntiles && j < prefetch && wp.t < wp.nt - 1; ++j) {
                 const int tok = wp.t * kTileKeys;
-#pragma unroll
-                for (int dp = 0; dp < (KF8 ? 1 : Lt::kPanels); ++dp)
-                    tma_prefetch_5d(&tm_k, dp * 64, wp.h, tok, wp.b, p.key_slab);
-#pragma unroll
-                for (int dp = 0; dp < (VF8 ? 1 : Lt::kPanels); ++dp)
-                    tma_prefetch_5d(&tm_v, dp * 64, wp.h, tok, wp.b, p.value_slab);
+                if (KF8) {
+                    tma_prefetch_5d(&tm_k, 0, wp.h, tok, wp.b, p.key_slab);
+                } else if (j == 0) {  // (bf16: the step's two tiles at once)
+                    tma_prefetch_5d(&tm_k2, 0, tok, 0, wp.h, p.key_slab * p.B + wp.b);
+                }
+                if (VF8)
+                    tma_prefetch_5d(&tm_v, 0, wp.h, tok, wp.b, p.value_slab);
+                else
+                    tma_prefetch_5d(&tm_v, 0, tok, 0, wp.h, p.value_slab * p.B + wp.b);
                 ++wp.t;  // stays inside the pair: its last (block) tile ends the loop
             }
         }
     }
 
-    // Producer state and one step of its loop (tile j of the range): the
-    // first steps may run before the lengths are checked (below).
+    // Loads, issued by two warps, each walking the range on its own: the S warp
+    // those of K (a slot is refilled as soon as the S that read it is done,
+    // whatever V waits for), the producer warp the query rows and V.  The
+    // first kFirstSteps steps' loads are all the producer's, in the order in
+    // which they are needed (an SM takes about 64 bytes a cycle from L2: issued
+    // by two warps at once, the first K came 0.6 us later), and may go out
+    // before the lengths are checked (below).
+    constexpr int kFirstSteps = 2;
+    static_assert(KS >= kFirstSteps && VS >= 2 * kFirstSteps, "first loads never wait");
     Walk wl = w0;
-    int qseg = -1;
-    long long nblk = 0;           // (kQSplit) block tiles whose keys were issued
-    long long issued = 0, j = 0;  // tiles whose loads were issued; next tile
+    Seg sg = {0, 0, 0, 0, false};
+    int qseg = -1, si = 0;         // segment, step of the segment
+    int done = 0, loads = 0, kloads = 0;  // tiles of past segments; V and K slots filled
+    Ring<KS> rk;
+    Ring<VS> rv;
     bool ok = true;
     uint64_t policy = 0;
-    if (warp == kProducerWarp)
+    if (warp == kProducerWarp || warp == kSWarp)
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-    auto produce = [&]() {
-        if (j == 0 || wl.t == 0) {  // the segment's query rows
-            ++qseg;
-            const int qb = qseg & 1;
-            if (qseg >= 2)
-                ok = ok && wait(b_qempty + 8 * qb, (uint32_t)(((qseg - 2) >> 1) & 1),
-                                abort_flag, p.status);
-            if (ok && elect_one()) {
-                const uint32_t full = b_qfull + 8 * qb;
-                const uint32_t dst = sbase + Lt::kQOff + qb * Lt::kQBytes;
-                // (NC > 1) copy c at rows c 64 / NC
-                mbar_arrive_expect_tx(full, NC * Lt::kPanels * p.rows_max * 128);
-#pragma unroll
-                for (int dp = 0; dp < Lt::kPanels; ++dp)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c)
-                        tma_4d(dst + dp * (kRows * 128) + c * (kRows / NC * 128), &tm_q, full,
-                               dp * 64, wl.h * p.G, 0, wl.b);
-            }
+    auto next_step = [&]() {
+        if (++si == sg.steps) {
+            si = 0;
+            done += sg.tiles;
+            walk_segment(p, wl, sg);
         }
-        const int s = (int)(j % kStages);
-        if (j >= kStages)
-            ok = ok && wait(b_empty + 8 * s, (uint32_t)(((j - kStages) / kStages) & 1),
-                            abort_flag, p.status);
-        const bool blk = wl.t == wl.nt - 1;
-        // (kQSplit) the block-key buffer is free once the S of the last block tile is done
-        if (kQSplit && blk && nblk >= 1)
-            ok = ok && wait(b_bkfree, (uint32_t)((nblk - 1) & 1), abort_flag, p.status);
-        if (ok && elect_one()) {
-            const uint32_t full = b_full + 8 * s;
-            const uint32_t kdst = sbase + Lt::kStagesOff + s * Lt::kStageBytes;
-            const uint32_t vdst = kdst + Lt::kKBytes;
-            if (wl.t < wl.nt - 1) {
-                const int tok = wl.t * kTileKeys;
-                mbar_arrive_expect_tx(full, Lt::kStageBytes);
-                // an e4m3 tile is one {D, 1, 64} box, a bf16 tile D / 64 swizzled panels
-                if (KF8) {
-                    tma_5d(kdst, &tm_k, full, 0, wl.h, tok, wl.b, p.key_slab, policy);
-                } else {
+    };
+    auto step_tile0 = [&]() {
+        return kConv && 2 * si >= sg.pairs ? wl.nt - 1 : wl.t + 2 * si;
+    };
+    // K of the current step, into a free slot
+    auto load_k = [&]() {
+        const int n = step_tiles(sg, si), t0 = step_tile0();
+        if (elect_one()) {
+            const uint32_t full = b_kfull + 8 * rk.slot;
+            const uint32_t dst = sbase + rk.slot * Lt::kKBytes;
+            const bool blk_last = t0 + n == wl.nt;  // the step's last tile is the block tile
+            mbar_arrive_expect_tx(full, KF8 ? (blk_last ? Lt::kTileBytes : n * (Lt::kKBytes / 2))
+                                            : n * Lt::kTileBytes);
+            if (t0 + 1 < wl.nt - 1 && n == 2) {  // two prefix tiles
+                if (KF8)
+                    tma_5d(dst, &tm_k2, full, 0, wl.h, t0 * kTileKeys, wl.b, p.key_slab, policy);
+                else
+                    tma_5d(dst, &tm_k2, full, 0, t0 * kTileKeys, 0, wl.h, p.key_slab * p.B + wl.b,
+                           policy);
+            } else {
+                for (int h = 0; h < n; ++h) {
+                    const int t = t0 + h;
+                    if (KF8 && t < wl.nt - 1) {
+                        tma_5d(dst + h * (Lt::kKBytes / 2), &tm_k, full, 0, wl.h, t * kTileKeys,
+                               wl.b, p.key_slab, policy);
+                        continue;
+                    }
 #pragma unroll
-                    for (int dp = 0; dp < Lt::kPanels; ++dp)
-                        tma_5d(kdst + dp * 8192, &tm_k, full, dp * 64, wl.h, tok, wl.b,
-                               p.key_slab, policy);
-                }
-                if (VF8) {
-                    tma_5d(vdst, &tm_v, full, 0, wl.h, tok, wl.b, p.value_slab, policy);
-                } else {
-#pragma unroll
-                    for (int dp = 0; dp < Lt::kPanels; ++dp)
-                        tma_5d(vdst + dp * 8192, &tm_v, full, dp * 64, wl.h, tok, wl.b,
-                               p.value_slab, policy);
-                }
-            } else if (kQSplit) {  // the block's own K (bf16) into its buffer, V into the stage
-                mbar_arrive_expect_tx(full, 2 * Lt::kTileBytes);
-#pragma unroll
-                for (int dp = 0; dp < Lt::kPanels; ++dp) {
-                    tma_4d(sbase + Lt::kBlkKOff + dp * 8192, &tm_kb, full, dp * 64, wl.h, 0,
-                           wl.b);
-                    tma_4d(vdst + dp * 8192, &tm_vb, full, dp * 64, wl.h, 0, wl.b);
-                }
-            } else {  // the block's own K / V (bf16): the operands read from the
-                      // stage; ring-slot operands are loaded by the conversion warps
-                mbar_arrive_expect_tx(full, (KF8 ? 0 : Lt::kTileBytes) +
-                                                (VF8 ? 0 : Lt::kTileBytes));
-#pragma unroll
-                for (int dp = 0; dp < Lt::kPanels; ++dp) {
-                    if (!KF8) tma_4d(kdst + dp * 8192, &tm_kb, full, dp * 64, wl.h, 0, wl.b);
-                    if (!VF8) tma_4d(vdst + dp * 8192, &tm_vb, full, dp * 64, wl.h, 0, wl.b);
+                    for (int dp = 0; dp < Lt::kPanels; ++dp) {
+                        // (e4m3 keys: the bf16 block tile, of 64-key panels)
+                        const uint32_t at = dst + dp * (KF8 ? 8192 : 16384) + h * 8192;
+                        if (t < wl.nt - 1)
+                            tma_5d(at, &tm_k, full, 0, t * kTileKeys, dp, wl.h,
+                                   p.key_slab * p.B + wl.b, policy);
+                        else
+                            tma_4d(at, &tm_kb, full, dp * 64, wl.h, 0, wl.b);
+                    }
                 }
             }
         }
         __syncwarp();
-        if (ok && kQSplit && blk) ++nblk;
-        if (ok) issued = j + 1;
-        walk_next(p, wl);
-        ++j;
+        ++kloads;
+        rk.next();
+    };
+    // the current step's V and, with its segment's first, the query rows
+    // (first = true: and its K, between the two)
+    auto load_qv = [&](bool first) {
+        if (si == 0) {
+            sg = segment<kConv>(wl, ntiles - done);
+            ++qseg;
+            const int qb = qseg & 1;
+            if (qseg >= 2) ok = ok && await(b_qempty, qb, (qseg - 2) >> 1);
+            if (ok && elect_one()) {
+                const uint32_t full = b_qfull + 8 * qb;
+                const uint32_t dst = sbase + Lt::kQOff + qb * Lt::kQBytes;
+                mbar_arrive_expect_tx(full, Lt::kPanels * p.rows_max * 128);
+#pragma unroll
+                for (int dp = 0; dp < Lt::kPanels; ++dp)
+                    tma_4d(dst + dp * (N * 128), &tm_q, full, dp * 64, wl.h * p.G, 0, wl.b);
+            }
+        }
+        if (first) load_k();
+        const int n = step_tiles(sg, si), t0 = step_tile0();
+        for (int h = 0; h < n; ++h) {
+            const int t = t0 + h;
+            // (e4m3 values) the conversion warps load a block tile's V
+            if (VF8 && t == wl.nt - 1) break;
+            if (loads >= VS) ok = ok && await(b_vempty, rv.slot, rv.parity ^ 1);
+            if (ok && elect_one()) {
+                const uint32_t full = b_vfull + 8 * rv.slot;
+                const uint32_t dst = sbase + Lt::kVOff + rv.slot * Lt::kVBytes;
+                mbar_arrive_expect_tx(full, Lt::kVBytes);
+                if (VF8) {
+                    tma_5d(dst, &tm_v, full, 0, wl.h, t * kTileKeys, wl.b, p.value_slab, policy);
+                } else if (t < wl.nt - 1) {
+                    tma_5d(dst, &tm_v, full, 0, t * kTileKeys, 0, wl.h, p.value_slab * p.B + wl.b,
+                           policy);
+                } else {
+#pragma unroll
+                    for (int dp = 0; dp < Lt::kPanels; ++dp)
+                        tma_4d(dst + dp * 8192, &tm_vb, full, dp * 64, wl.h, 0, wl.b);
+                }
+            }
+            __syncwarp();
+            if (!ok) break;
+            ++loads;
+            rv.next();
+        }
+        next_step();
     };
 
     // every input (and the workspace) may be written by the previous kernel
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the first loads of the speculative plan go out while the lengths are
-    // checked (no step here waits: fresh stages and query buffers only)
-    if (spec && warp == kProducerWarp)
-        while (j < ntiles && j < kStages && ok && !((j == 0 || wl.t == 0) && qseg + 1 >= 2) &&
-               !(kQSplit && wl.t == wl.nt - 1 && nblk >= 1))
-            produce();
+    // checked (no step here waits: fresh slots and query buffers only)
+    auto first_loads = [&]() {
+        for (int u = 0; u < kFirstSteps && done < ntiles; ++u) load_qv(true);
+    };
+    if (spec && warp == kProducerWarp) first_loads();
     {
         const int P1 = lane0 < p.B ? len_cg(p.prefix_len, lane0, p.capacity) : 0;
         const int T1 = lane0 < p.B ? len_cg(p.block_len, lane0, p.max_block) : 0;
         if (!(spec && __all_sync(kFull, P1 == sP && T1 == sT))) {  // the same in every warp
             if (spec) {  // loads issued under the stale plan land, then the barriers restart
                 if (warp == kProducerWarp) {
-                    for (long long t = 0; t < issued; ++t)
-                        wait(b_full + 8 * (int)t, 0u, abort_flag, p.status);
-                    for (int q = 0; q <= qseg; ++q) wait(b_qfull + 8 * q, 0u, abort_flag, p.status);
+                    for (int s = 0; s < kloads; ++s) await(b_kfull, s, 0);
+                    for (int s = 0; s < loads; ++s) await(b_vfull, s, 0);
+                    for (int q = 0; q <= qseg; ++q) await(b_qfull, q, 0);
                 }
                 __syncthreads();
                 if (threadIdx.x == 0) init_bars();
@@ -1121,11 +873,12 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
             }
             lo = hi = 0;
             w0 = {0, 0, 0, 1, 0, 0};
-            ntiles = plan(p, P1, T1, lo, hi, w0) ? hi - lo : 0;
+            ntiles = plan(p, P1, T1, lo, hi, w0) ? (int)(hi - lo) : 0;
             wl = w0;
             qseg = -1;
-            nblk = 0;
-            issued = j = 0;
+            si = done = loads = kloads = 0;
+            rk = Ring<KS>();
+            rv = Ring<VS>();
             ok = true;
         }
     }
@@ -1136,139 +889,610 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                 atomicOr(p.status, kStatusClamped);
     // an empty range (only when N < C) runs no loop below
 
-    // the last loads each issuing thread started, for the abort path's drain
-    long long drain_tiles = 0, drain_copy = -1;
-    int drain_qseg = -1;
+    // keys of a segment's first reference
+    auto ref_keys = [&](const Walk &w) { return VF8 || w.nt <= kRefTiles ? kRefKeys : kRefKeys / 2; };
+
+    int drain_copy = -1;  // the last copy a conversion warp started, for the abort path's drain
     if (warp == kProducerWarp) {
         // ================================ producer ===============================
-        // Warp-uniform loop; one elected lane issues.  Stage s is reused once
-        // the P V that read it has completed (the P V warp commits empty[s]);
-        // a query buffer once the last S of the segment before last completed.
-        while (j < ntiles && ok) produce();
-        drain_tiles = issued;
-        drain_qseg = qseg;
-    } else if (warp == kMmaWarp || warp == kSWarp) {
-        // ================================== MMA ==================================
-        // Two issuing warps, each blocking on its own in-order stream: P V of
-        // tile k once its P is in shared memory (pready), and S of tile kn once
-        // its K has landed (or been widened), its segment's queries are in and
-        // TMEM buffer kn % kSBufs has been read by the softmax warps (sfree).
-        const uint32_t id_s = idesc(kRows, kTileKeys, 0, 0);
-        const uint32_t id_pv = idesc(kRows, D, 0, 1);
+        // Warp-uniform loop; one elected lane issues.  A V slot is reused once
+        // the P V (or the widening) that read it has completed, a query buffer
+        // once the last S of the segment before last has (and the softmax
+        // warps have read its scales).
+        if (kloads == 0) first_loads();  // (not spec, or the lengths had changed)
+        while (done < ntiles && ok) load_qv(false);
+    } else if (warp == kSWarp) {
+        // =============================== S^T = K Q^T =============================
+        const uint32_t id_s = idesc(128, N, 0, 0);
+        const uint32_t id_s8 = idesc_e4m3(128, N);
         // descriptors are affine in the address: build each base once and add
-        // (byte offset >> 4) for buffers and k-steps
-        const uint64_t dq0 = sdesc(sbase + Lt::kQOff, 16, 1024);
-        const uint64_t dk0 = sdesc(k_src(0, 0), 16, 1024);
-        // (kQSplit) e4m3 operands: query parts hi / lo of buffer b at
-        // kQ8Off + (2 b + part) kQ8Bytes, prefix keys in the stage, block keys (bf16)
-        const uint32_t id_s8 = idesc_e4m3(kRows, kTileKeys);
-        const uint64_t dq8 = sdesc(sbase + Lt::kQ8Off, 16, 1024);
-        const uint64_t dk8 = sdesc(sbase + Lt::kStagesOff, 16, 1024);
-        const uint64_t dkb = sdesc(sbase + Lt::kBlkKOff, 16, 1024);
-        const uint64_t dv0 = sdesc(v_src(0, 0), 8192, 1024);
-        const uint64_t dp0 = sdesc(sbase + Lt::kPOff, 16, 1024);
-        // rounded row sums: D[64][8] += P[64][64] ones[8][64]^T, column 0 = sum of P
-        const uint64_t d1 = sdesc(sbase + Lt::kOnesOff, 16, 1024);
-        const uint32_t id_l = idesc(kRows, 8, 0, 0);
-        bool ok = true;
-        if (warp == kSWarp) {
-            Walk wsn = w0;
-            int qseg = -1, qcur = 0;
-            for (long long kn = 0; kn < ntiles && ok; ++kn) {
-                if (kn == 0 || wsn.t == 0) {
-                    ++qseg;
-                    qcur = qseg & 1;
-                    ok = ok && wait(b_qfull + 8 * qcur, (uint32_t)((qseg >> 1) & 1), abort_flag,
-                                    p.status);
-                    // (kQSplit) and split into its e4m3 parts
-                    if (kQSplit)
-                        ok = ok && wait(b_qsplit + 8 * qcur, (uint32_t)((qseg >> 1) & 1),
-                                        abort_flag, p.status);
+        // (byte offset >> 4) for slots, panels and k-steps
+        const uint64_t dk = sdesc(sbase, 16, 1024, kSw128);
+        const uint64_t dq = sdesc(sbase + Lt::kQOff, 16, 1024, kSw128);
+        const uint64_t dk8 = sdesc(sbase, 16, 8 * D, D == 128 ? kSw128 : kSw64);
+        const uint64_t dq8 = sdesc(sbase + Lt::kQ8Off, 16, 8 * D, D == 128 ? kSw128 : kSw64);
+        // Of a segment's first step, the scores of its first keys are also formed the
+        // other way round (rows in lanes: M = 64), where each row's maximum, the
+        // first reference, is one thread's.
+        // The walk over the steps that the producer loaded, then K of the slots
+        // left.  e4m3 keys: while the query rows are split; else the first S first.
+        auto start_loads = [&]() {
+            for (int u = 0; done < ntiles && u < KS; ++u) {
+                if (si == 0) sg = segment<kConv>(wl, ntiles - done);
+                if (u < kFirstSteps) {
+                    ++kloads;
+                    rk.next();
+                } else {
+                    load_k();
                 }
-                const int s = (int)(kn % kStages);
-                // the tile's K and V: landed, and widened if stored as e4m3 (kQSplit:
-                // the e4m3 keys are read as they are)
-                if (Lt::kConv && !kQSplit)
-                    ok = ok && wait(b_cready + 8 * (int)(kn % kSlots),
-                                    (uint32_t)((kn / kSlots) & 1), abort_flag, p.status);
-                else
-                    ok = ok && wait(b_full + 8 * s, (uint32_t)((kn / kStages) & 1), abort_flag,
-                                    p.status);
-                if (kn >= kSBufs)
-                    ok = ok && wait(b_sfree + 8 * (int)(kn % kSBufs),
-                                    (uint32_t)(((kn - kSBufs) / kSBufs) & 1), abort_flag,
-                                    p.status);
+                next_step();
+            }
+        };
+        if (KF8) start_loads();
+        Walk w = w0;
+        Ring<KS> ru;          // slot being read
+        Ring<kSBufs> rs, rf;  // rf: the last segment's first step, kf
+        for (int past = 0, seg = 0, k = 0, kf = 0; past < ntiles && ok; ++seg) {
+            const Seg sc = segment<kConv>(w, ntiles - past);
+            const int qb = seg & 1;
+            const uint32_t id_r = idesc(64, ref_keys(w), 0, 0), id_r8 = idesc_e4m3(64, ref_keys(w));
+            ok = await(b_qfull, qb, seg >> 1);
+            if (KF8) ok = ok && await(b_qsplit, qb, seg >> 1);
+            for (int i = 0; i < sc.steps && ok; ++i, ++k) {
+                ok = await(b_kfull, ru.slot, ru.parity);
+                // the softmax has read the scores of step k - kSBufs
+                if (k >= kSBufs) ok = ok && await(b_sfree, rs.slot, rs.parity ^ 1);
+                // and the last segment's reference scores: implied unless its
+                // first step is a later one (whose buffer then has no later
+                // phase, so that the parity is exact)
+                if (i == 0 && seg > 0 && k - kf < kSBufs)
+                    ok = ok && await(b_sfree, rf.slot, rf.parity);
                 if (!ok) break;
-                const bool blk_tile = wsn.t == wsn.nt - 1;
-                const bool seg_end = blk_tile || (kn + 1 == ntiles);
                 fence_after();
                 if (elect_one()) {
-                    const uint32_t dS = tmem + (uint32_t)((kn % kSBufs) * kTileKeys);
-                    if (kQSplit && !blk_tile) {
-                        // S = hi K^T + lo K^T: 2 x 4 MMAs of 32 e4m3 elements (32 bytes)
-                        const uint64_t ah = dq8 + (uint64_t)((2 * qcur * Lt::kQ8Bytes) >> 4);
-                        const uint64_t al = ah + (uint64_t)(Lt::kQ8Bytes >> 4);
-                        const uint64_t b0 = dk8 + (uint64_t)((s * Lt::kStageBytes) >> 4);
+                    const uint32_t dS = tmem + (uint32_t)(rs.slot * N), dR = tmem + Lt::kRefCol;
+                    const uint32_t slot = (uint32_t)(ru.slot * Lt::kKBytes) >> 4;
+                    // hi K^T, then lo K^T (, then lo2 K^T), 32 elements (32 bytes) per
+                    // MMA (the third part is e5m2: B of S^T, A of the reference scores);
+                    // bf16: panel kk / 4, then 16 elements within the 128-byte row
+                    const bool f8 = KF8 && 2 * i < sc.pairs;
+                    auto key8 = [&](int kk) { return dk8 + (uint64_t)(slot + kk % (D / 32) * 2); };
+                    auto qry8 = [&](int kk) {
+                        return dq8 + (uint64_t)((kk / (D / 32) * Lt::kQ8Bytes + kk % (D / 32) * 32) >> 4);
+                    };
+                    auto key16 = [&](int kk) {
+                        return dk + (uint64_t)(slot + (((kk >> 2) * (KF8 ? 8192 : 16384) +
+                                                        (kk & 3) * 32) >> 4));
+                    };
+                    auto qry16 = [&](int kk) {
+                        return dq + (uint64_t)((qb * Lt::kQBytes + (kk >> 2) * (N * 128) +
+                                                (kk & 3) * 32) >> 4);
+                    };
+                    if (i == 0) {  // first: the softmax takes the references meanwhile
+                        if (f8) {
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            mma_e4m3(dS, ah + (uint64_t)(kk * 2), b0 + (uint64_t)(kk * 2), id_s8,
-                                     kk > 0);
+                            for (int kk = 0; kk < Lt::kParts * (D / 32); ++kk)
+                                mma_f8(dR, qry8(kk), key8(kk),
+                                       kk / (D / 32) < 2 ? id_r8 : id_r8 | 1u << 7, kk > 0);
+                        } else {
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            mma_e4m3(dS, al + (uint64_t)(kk * 2), b0 + (uint64_t)(kk * 2), id_s8,
-                                     1u);
+                            for (int kk = 0; kk < D / 16; ++kk)
+                                mma(dR, qry16(kk), key16(kk), id_r, kk > 0);
+                        }
+                        mma_commit(b_rready);
+                    }
+                    if (f8) {
+#pragma unroll
+                        for (int kk = 0; kk < Lt::kParts * (D / 32); ++kk)
+                            mma_f8(dS, key8(kk), qry8(kk),
+                                   kk / (D / 32) < 2 ? id_s8 : id_s8 | 1u << 10, kk > 0);
                     } else {
-                        const uint64_t a0 = dq0 + (uint64_t)((qcur * Lt::kQBytes) >> 4);
-                        const uint64_t b0 =
-                            kQSplit ? dkb
-                                    : dk0 + (uint64_t)((k_src(s, kn) - k_src(0, 0)) >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk) {
-                            // panel kk / 4, then 16 elements (32 bytes) within the 128-byte row
-                            const uint32_t qoff =
-                                ((kk >> 2) * (kRows * 128) + (kk & 3) * 32) >> 4;
-                            const uint32_t koff = ((kk >> 2) * 8192 + (kk & 3) * 32) >> 4;
-                            mma(dS, a0 + qoff, b0 + koff, id_s, kk > 0);
+                        for (int kk = 0; kk < D / 16; ++kk)
+                            mma(dS, key16(kk), qry16(kk), id_s, kk > 0);
+                    }
+                    mma_commit(b_sready + 8 * rs.slot);
+                    mma_commit(b_kempty + 8 * ru.slot);
+                    if (i == sc.steps - 1) mma_commit(b_qempty + 8 * qb);
+                }
+                __syncwarp();
+                // fill the slots not used yet, refill this one once these S are done
+                if (!KF8 && k == 0) start_loads();
+                if (done < ntiles) {  // refill the slot once these S are done
+                    ok = await(b_kempty, ru.slot, ru.parity);
+                    if (ok) {
+                        if (si == 0) sg = segment<kConv>(wl, ntiles - done);
+                        load_k();
+                        next_step();
+                    }
+                }
+                if (i == 0) {
+                    rf = rs;
+                    kf = k;
+                }
+                ru.next();
+                rs.next();
+            }
+            past += sc.tiles;
+            walk_segment(p, w, sc);
+        }
+    } else if (warp == kMmaWarp) {
+        // ========================= O^T += V^T P^T, l += 1 P^T ====================
+        // A is MN-major: V as it lies (dims contiguous).  D = 64: M = 128, the
+        // second 64 rows of A are ones, so lanes 64.. accumulate the row sums
+        // of P as rounded; D = 128: they take MMAs of their own, with the ones
+        // in tensor memory (shared memory is the scarcer port).
+        const uint64_t dp = sdesc(sbase + Lt::kPOff, 16, 16 * N, N == 64 ? kSw128 : N == 32 ? kSw64 : kSw32);
+        const uint32_t vbase = sbase + (VF8 ? Lt::kWOff : Lt::kVOff);
+        constexpr int kVStride = VF8 ? Lt::kTileBytes : Lt::kVBytes;
+        const uint32_t b_v = VF8 ? b_wready : b_vfull, b_vdone = VF8 ? b_wfree : b_vempty;
+        const uint32_t dO = tmem + Lt::kOCol;
+        Walk w = w0;
+        Ring<VF8 ? WS : VS> rv;
+        bool ok = true;
+        for (int done = 0, k = 0; done < ntiles && ok;) {
+            const Seg sg = segment<kConv>(w, ntiles - done);
+            // 16-key groups of the last tile that P V reads, and of a last step of it alone
+            const int last_groups = (tile_keys(w, w.t + sg.tiles - 1) + 15) >> 4;
+            for (int i = 0; i < sg.steps; ++i, ++k) {
+                const int n = step_tiles(sg, i);
+                const bool last = i == sg.steps - 1;
+                // (a partly filled prefix tile before a block step of its own is all zeros past its keys)
+                const int groups = !last ? 4 * n : n == 2 ? 4 + last_groups : max(last_groups, 1);
+                const bool f16 = VF8 && 2 * i < sg.pairs;  // widened values: f16
+                const uint32_t id_pv = f16 ? idesc_f16(128, N, 1, 1) : idesc(128, N, 1, 1);
+                const uint32_t id_l = f16 ? idesc_f16(128, N, 0, 1) : idesc(128, N, 0, 1);
+                const uint32_t ones = sbase + Lt::kOnesOff + (f16 ? 2048 : 0);
+                const Ring<VF8 ? WS : VS> r0 = rv;
+                ok = await(b_v, rv.slot, rv.parity);
+                rv.next();
+                const int slot1 = rv.slot;
+                if (n == 2) {
+                    ok = ok && await(b_v, rv.slot, rv.parity);
+                    rv.next();
+                }
+                ok = ok && await(b_pready, k & 1, k >> 1);
+                if (!ok) break;
+                fence_after();
+                if (elect_one()) {
+                    const uint64_t b0 = dp + (uint64_t)(((k & 1) * Lt::kPBytes) >> 4);
+                    const bool acc0 = i > 0;
+                    const uint32_t va0 = vbase + r0.slot * kVStride, va1 = vbase + slot1 * kVStride;
+#pragma unroll
+                    for (int g = 0; g < 8; ++g) {
+                        if (g >= groups) break;
+                        const uint32_t va = (g < 4 ? va0 : va1) + (g & 3) * 2048;
+                        mma(dO, sdesc(va, D == 128 ? 8192 : ones - va, 1024, kSw128),
+                            b0 + (uint64_t)((g * 32 * N) >> 4), id_pv, acc0 || g > 0);
+                    }
+                    if (D == 128) {
+                        const uint32_t a = tmem + Lt::kOnesCol + (f16 ? 8 : 0);
+#pragma unroll
+                        for (int g = 0; g < 8; ++g) {
+                            if (g >= groups) break;
+                            mma_ta(tmem + Lt::kLCol, a, b0 + (uint64_t)((g * 32 * N) >> 4), id_l,
+                                   acc0 || g > 0);
                         }
                     }
-                    mma_commit(b_sready + 8 * (int)(kn % kSBufs));
-                    if (KF8 && !kQSplit) mma_commit(b_kfree + 8 * (int)(kn % kSlots));
-                    if (kQSplit && blk_tile) mma_commit(b_bkfree);
-                    if (seg_end) mma_commit(b_qempty + 8 * qcur);
+                    mma_commit(b_pvdone + 8 * (k & 1));
+                    mma_commit(b_vdone + 8 * r0.slot);
+                    if (n == 2) mma_commit(b_vdone + 8 * slot1);
                 }
                 __syncwarp();
-                walk_next(p, wsn);
             }
-        } else {
-            Walk wm = w0;
-            for (long long k = 0; k < ntiles && ok; ++k) {
-                const bool first = (k == 0) || (wm.t == 0);
-                ok = wait(b_pready + 8 * (int)(k & 1), (uint32_t)((k >> 1) & 1), abort_flag,
-                          p.status);
-                if (!ok) break;
-                fence_after();
-                if (elect_one()) {
-                    const int s = (int)(k % kStages);
-                    const uint64_t a0 = dp0 + (uint64_t)(((k & 1) * Lt::kPBytes) >> 4);
-                    const uint64_t b0 = dv0 + (uint64_t)((v_src(s, k) - v_src(0, 0)) >> 4);
-                    const uint32_t dO = tmem + kSBufs * kTileKeys;
-#pragma unroll
-                    for (int kk = 0; kk < kTileKeys / 16; ++kk)
-                        mma(dO, a0 + (uint64_t)((kk * 32) >> 4),
-                            b0 + (uint64_t)((kk * 2048) >> 4), id_pv,
-                            (!first || kk > 0) ? 1u : 0u);
-#pragma unroll
-                    for (int kk = 0; kk < kTileKeys / 16; ++kk)
-                        mma(dO + D, a0 + (uint64_t)((kk * 32) >> 4), d1 + (uint64_t)((kk * 32) >> 4),
-                            id_l, (!first || kk > 0) ? 1u : 0u);
-                    mma_commit(b_pvdone + 8 * (int)(k & 1));
-                    mma_commit(b_empty + 8 * s);
-                    if (VF8) mma_commit(b_vfree + 8 * (int)(k % kSlots));
-                }
-                __syncwarp();
-                walk_next(p, wm);
-            }
+            done += sg.tiles;
+            walk_segment(p, w, sg);
         }
+    } else if (kConv && warp >= kConvWarp0) {
+        // ==================== query split, e4m3 -> f16 values ====================
+        const int ct = threadIdx.x - kConvWarp0 * 32;
+        float *qsc = reinterpret_cast<float *>(sm + Lt::kQscOff);
+        Walk w = w0;
+        int seg = -1, vt = 0;
+        for (int j = 0; j < ntiles; ++j) {
+            if (KF8 && (j == 0 || w.t == 0)) {
+                // The parts are overwritten once the last segment's S are done
+                // (a step or two before the softmax ends it), the scales of
+                // buffer b once the segment before last's are read: qempty.
+                ++seg;
+                const int qb = seg & 1;
+                if (seg >= 1 && !await(b_qempty, qb ^ 1, (seg - 1) >> 1)) break;
+                if (!await(b_qfull, qb, seg >> 1)) break;
+                split_q<D, N, Lt::kParts>(sbase + Lt::kQOff + qb * Lt::kQBytes,
+                                          sbase + Lt::kQ8Off, qsc + qb * N, p.scale_log2, ct);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(b_qsplit + 8 * qb);
+            }
+            if (VF8) {
+                const uint32_t wr = b_wready + 8 * (j % WS);
+                const uint32_t dst = sbase + Lt::kWOff + (j % WS) * Lt::kTileBytes;
+                if (j >= WS && !await(b_wfree, j % WS, j / WS - 1)) break;
+                if (w.t == w.nt - 1) {
+                    // the block's V is bf16: one lane loads it into the slot
+                    // with a copy that completes on wready itself
+                    if (warp == kConvWarp0) {
+                        if (elect_one()) {
+                            mbar_arrive_expect_tx(wr, Lt::kTileBytes);
+#pragma unroll
+                            for (int dp = 0; dp < Lt::kPanels; ++dp)
+                                tma_4d(dst + dp * 8192, &tm_vb, wr, dp * 64, w.h, 0, w.b);
+                        }
+                        drain_copy = j;
+                    } else if (lane == 0) {
+                        mbar_arrive(wr);
+                    }
+                    __syncwarp();
+                } else {
+                    const int vs = vt % VS;
+                    if (!await(b_vfull, vs, vt / VS)) break;
+                    widen_tile<D>(sbase + Lt::kVOff + vs * Lt::kVBytes, dst, tile_keys(w, w.t), ct);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(wr);
+                        mbar_arrive(b_vempty + 8 * vs);
+                    }
+                    ++vt;
+                }
+            }
+            walk_next(p, w);
+        }
+    } else if (warp < kSoftWarps) {
+        // ================================ softmax ================================
+        // Thread j of a group holds key j of the step: its group's kCols scores
+        // of that lane of S^T.  With N = 64 two groups take 32 columns each,
+        // independent of one another up to P (two warps per scheduler, which
+        // hide each other's latencies; one group of 64 columns needed 255
+        // registers and was slower on every 64-column case).
+        constexpr int NC = Lt::kCols;
+        const int group = Lt::kGroups == 1 ? 0 : warp >> 2, key = threadIdx.x & 127;
+        const int half = key >> 6, kidx = key & 63;  // tile of the step, key of the tile
+        const int col0 = group * NC;
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        // per query row, this group's: -reference, rescale factor, per-warp
+        // partials [4][N], rounded row sum (shared memory); -reference and
+        // score scale in every lane of tensor memory
+        const uint32_t rows = sbase + Lt::kNmOff + col0 * 4;
+        const uint32_t nm_sm = rows, al_sm = rows + (Lt::kAlphaOff - Lt::kNmOff),
+                       red_sm = rows + (Lt::kRedOff - Lt::kNmOff),
+                       lr_sm = rows + (Lt::kLrOff - Lt::kNmOff);
+        const uint32_t pkey = sbase + Lt::kPOff + key * (2 * N);
+        const int pswz = N == 64 ? key & 7 : N == 32 ? (key >> 1) & 3 : (key >> 2) & 1;
+        const uint32_t nm_t = tmem + lane_base + (uint32_t)(Lt::kNmCol + col0),
+                       sc_t = tmem + lane_base + (uint32_t)(Lt::kScCol + col0),
+                       sum_t = tmem + lane_base + (uint32_t)(Lt::kSumCol + col0);
+        Walk w = w0;
+        Ring<VF8 ? WS : VS> rv;
+        Ring<kSBufs> rs;
+        for (int done = 0, seg = 0, k = 0; done < ntiles; ++seg) {
+        const Seg sg = segment<kConv>(w, ntiles - done);
+        const int rows_active = p.G * w.T - col0;
+        const uint32_t sc_row = rows + (Lt::kQscOff - Lt::kNmOff) + (seg & 1) * N * 4;
+        if (KF8) {
+            await(b_qsplit, seg & 1, seg >> 1);
+            row_values_to_tmem<NC>(sc_row, sc_t);
+            // the scales are read: their buffer may take the segment after next's
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b_qempty + 8 * (seg & 1));
+        }
+        for (int i = 0; i < sg.steps; ++i, ++k, rs.next()) {
+            const bool first = i == 0;
+            const bool last = i == sg.steps - 1;
+            const bool full = i < sg.nfull;                  // every key visible to every row
+            const bool f8s = KF8 && 2 * i < sg.pairs;        // the scores carry a scale per row
+            const int n = step_tiles(sg, i);
+            const int t0 = kConv && 2 * i >= sg.pairs ? w.nt - 1 : w.t + 2 * i;
+            // this key is visible to the rows from r0 on: all for a valid
+            // prefix key, rows i >= kidx (r / G >= kidx) for a block key
+            int r0 = 0;
+            if (!full) {
+                const int t = t0 + half;
+                const bool valid = half < n && kidx < tile_keys(w, t);
+                r0 = !valid ? N : t == w.nt - 1 ? kidx * p.G - col0 : 0;
+            }
+            // ---- scores of the step ----
+            const uint32_t s_addr = tmem + lane_base + (uint32_t)(rs.slot * N + col0);
+            float v[NC];
+            // v = score - reference (base 2), -inf where not visible
+            auto to_exponents = [&]() {
+                const float s0 = p.scale_log2;
+                if constexpr (KF8) {  // (three loads of 32 would spill)
+#pragma unroll
+                    for (int c = 0; c < NC; c += 16) {
+                        float m[16], s[16];
+                        tmem_ld_scores(s_addr + c, nm_t + c, sc_t + c, v + c, m, s);
+#pragma unroll
+                        for (int j = 0; j < 16; j += 2)
+                            fma2(v[c + j], v[c + j + 1], v[c + j], v[c + j + 1], f8s ? s[j] : s0,
+                                 f8s ? s[j + 1] : s0, m[j], m[j + 1]);
+                    }
+                } else {
+                    float m[NC];
+                    tmem_ld_two<NC>(s_addr, nm_t, v, m);
+#pragma unroll
+                    for (int j = 0; j < NC; j += 2)
+                        fma2(v[j], v[j + 1], v[j], v[j + 1], s0, s0, m[j], m[j + 1]);
+                }
+                if (!full)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) v[c] = c >= r0 ? v[c] : -INFINITY;
+            };
+            if (first) {  // the first reference, while S is formed
+                await(b_rready, 0, seg);
+                fence_after();
+                if ((warp & 3) * 16 >= col0 && (warp & 3) * 16 < col0 + NC) {
+                    float x[kRefKeys];
+                    tmem_ld<kRefKeys>(tmem + lane_base + (uint32_t)Lt::kRefCol, x);
+                    const int r = (warp & 3) * 16 + lane - col0;  // lanes < 16
+                    const int nv = min(ref_keys(w), tile_keys(w, t0));
+                    const int lim = t0 == w.nt - 1 ? min(nv, (r + col0) / p.G + 1) : nv;
+                    float m = -INFINITY;
+#pragma unroll
+                    for (int c = 0; c < kRefKeys; ++c) m = fmaxf(m, c < lim ? x[c] : -INFINITY);
+                    if (lane < 16) {
+                        m *= f8s ? lds(sc_row + 4 * r) : p.scale_log2;
+                        // a row with no finite score yet keeps a reference far below
+                        // any; rows past the block weigh nothing and never move it
+                        sts(nm_sm + 4 * r, r >= rows_active ? -INFINITY : m == -INFINITY ? kNoRef : -m);
+                    }
+                }
+                soft_sync(group);
+                row_values_to_tmem<NC>(nm_sm, nm_t);
+            }
+            await(b_sready, rs.slot, rs.parity);
+            fence_after();
+            to_exponents();
+            float m4[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) m4[j] = fmaxf(v[j], v[j + 4]);
+#pragma unroll
+            for (int c = 8; c < NC; c += 8)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) m4[j] = max3(m4[j], v[c + j], v[c + 4 + j]);
+            // a score far beyond its row's reference: the reference moves
+            const bool move =
+                soft_any(group, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) > (VF8 ? kRescaleF16 : kRescaleBf16));
+            const uint32_t pbuf = (uint32_t)((k & 1) * Lt::kPBytes);
+            if (move) {  // the same in all of the group's warps
+                // the rows' maxima over the step, through the P buffer (free once
+                // P V of step k - 2 is done)
+                if (k >= kPBufs) await(b_pvdone, k & 1, (k >> 1) - 1);
+#pragma unroll
+                for (int c = 0; c < NC; c += 16) {
+                    float m[16], s[16];
+                    tmem_ld_scores(s_addr + c, nm_t + c, (KF8 ? sc_t : nm_t) + c, v + c, m, s);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        v[c + j] = c + j >= r0 ? v[c + j] * (f8s ? s[j] : p.scale_log2) : -INFINITY;
+                }
+                lane_reduce<true, NC, N>(v, sbase + Lt::kPOff + pbuf, red_sm + (warp & 3) * N * 4, group, key);
+                soft_sync(group);
+                if (key < NC) {
+                    const int r = key;
+                    const uint32_t red = red_sm + 4 * r;
+                    const float m = fmaxf(fmaxf(lds(red), lds(red + 4 * N)),
+                                          fmaxf(lds(red + 8 * N), lds(red + 12 * N)));
+                    const float old = lds(nm_sm + 4 * r);
+                    float nm = old, alpha = 1.f;
+                    if (m + old > (VF8 ? kRescaleF16 : kRescaleBf16) && m != -INFINITY) {  // (old = -inf past the block)
+                        nm = -m;
+                        alpha = ex2(nm - old);
+                    }
+                    sts(nm_sm + 4 * r, nm);
+                    sts(al_sm + 4 * r, alpha);
+                }
+                soft_sync(group);
+                row_values_to_tmem<NC>(nm_sm, nm_t);
+                if (!first) {
+                    // O is stable once P V of step k - 1 is done
+                    await(b_pvdone, (k - 1) & 1, (k - 1) >> 1);
+                    fence_after();
+                    // the lane's sums, O and (D = 128) the rounded row sums
+                    tmem_wait_st();
+#pragma unroll 1
+                    for (int c = 0; c < (D == 128 ? 3 : 2) * NC; c += 16) {
+                        float o[16];
+                        const int at = c < NC       ? Lt::kSumCol
+                                       : c < 2 * NC ? Lt::kOCol - NC
+                                                    : Lt::kLCol - 2 * NC;
+                        const uint32_t ta = tmem + lane_base + (uint32_t)(at + col0 + c);
+                        tmem_ld<16>(ta, o);
+#pragma unroll
+                        for (int r = 0; r < 16; r += 4) {
+                            const float4 a = lds4(al_sm + 4 * ((c & (NC - 1)) + r));
+                            mul2(o[r], o[r + 1], o[r], o[r + 1], a.x, a.y);
+                            mul2(o[r + 2], o[r + 3], o[r + 2], o[r + 3], a.z, a.w);
+                        }
+                        tmem_st16(ta, o);
+                    }
+                    tmem_wait_st();
+                }
+                to_exponents();
+            }
+            // the scores are in registers: their buffer may take step k + kSBufs
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b_sfree + 8 * rs.slot);
+            // ---- P = 2^(s - m), as 16-bit floats into the P buffer ----
+#pragma unroll
+            for (int c = 0; c < NC; ++c) v[c] = ex2(v[c]);
+            uint32_t pk[NC / 2];
+            if (VF8 && 2 * i < sg.pairs) {
+#pragma unroll
+                for (int c = 0; c < NC / 2; ++c) pk[c] = pack_f16(v[2 * c], v[2 * c + 1]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < NC / 2; ++c) pk[c] = pack_bf16(v[2 * c], v[2 * c + 1]);
+            }
+            // the P buffer is free once P V of step k - 2, its last reader, is done
+            if (k >= kPBufs) await(b_pvdone, k & 1, (k >> 1) - 1);
+            const uint32_t prow = pkey + pbuf;
+#pragma unroll
+            for (int c = 0; c < NC / 8; ++c)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                                 prow + (((col0 / 8 + c) ^ pswz) << 4)),
+                             "r"(pk[4 * c]), "r"(pk[4 * c + 1]), "r"(pk[4 * c + 2]),
+                             "r"(pk[4 * c + 3])
+                             : "memory");
+            // keys past the end of a tile may hold anything: zero the V rows
+            // that P V reads (widened tiles hold zeros there)
+            for (int h = 0; h < n; ++h, rv.next()) {
+                if (full || (VF8 && 2 * i < sg.pairs)) continue;
+                const int nv = tile_keys(w, t0 + h);
+                // a tile with another after it is read whole, the last up to its 16-key group
+                const int end = !last || h + 1 < n ? kTileKeys : n == 1 && nv == 0 ? 16 : (nv + 15) & ~15;
+                if (nv >= end) continue;
+                await(VF8 ? b_wready : b_vfull, rv.slot, rv.parity);
+                const uint32_t vt = sbase + (VF8 ? Lt::kWOff + rv.slot * Lt::kTileBytes
+                                                 : Lt::kVOff + rv.slot * Lt::kVBytes);
+                const int chunks = (end - nv) * 8;
+                for (int c = threadIdx.x; c < chunks * Lt::kPanels; c += kSoftWarps * 32)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
+                                     vt + (c / chunks) * 8192 + nv * 128 + (c % chunks) * 16),
+                                 "r"(0u)
+                                 : "memory");
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b_pready + 8 * (k & 1));
+            // The lane's part of the sum of each row's fp32 weights (for the
+            // lse), after P has been handed on.  The sum of the weights as
+            // rounded for the P V product, used for the normalisation so that
+            // O / l is an exact convex combination of the values, is
+            // accumulated by the tensor core.
+            tmem_accumulate<NC>(sum_t, v, first);
+        }
+        // ---- end of segment: O / l and lse ----
+        --k;  // the last step
+        {
+            const bool whole = w.t == 0 && sg.blk;
+            const size_t slot = (size_t)(w.b * p.Hkv + w.h) + blockIdx.x;
+            // while P V of the last step runs, the sums over the keys (through
+            // the other P buffer)
+            if (k >= 1) await(b_pvdone, (k - 1) & 1, (k - 1) >> 1);
+            {
+                float l[NC];
+                tmem_wait_st();
+                tmem_ld<NC>(sum_t, l);
+                lane_reduce<false, NC, N>(l, sbase + Lt::kPOff + (uint32_t)((~k & 1) * Lt::kPBytes),
+                                          red_sm + (warp & 3) * N * 4, group, key);
+            }
+            await(b_pvdone, k & 1, k >> 1);
+            fence_after();
+            if (D == 64) {  // lanes 64.. hold the rounded row sums: to all through shared memory
+                if ((warp & 3) == 2) {
+                    float lr[NC];
+                    tmem_ld<NC>(tmem + lane_base + (uint32_t)(Lt::kOCol + col0), lr);
+                    if (lane == 0)
+#pragma unroll
+                        for (int r = 0; r < NC; r += 4)
+                            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(lr_sm + 4 * r),
+                                         "f"(lr[r]), "f"(lr[r + 1]), "f"(lr[r + 2]), "f"(lr[r + 3])
+                                         : "memory");
+                }
+                soft_sync(group);
+            }
+            // thread = dim (lane of O^T).  A whole pair's rows are staged as
+            // bf16 in the group's slice of the P buffer (read by no MMA until
+            // the group hands on its next P) and leave as 16-byte stores; a
+            // partial's fp32 rows go straight out, 128 bytes a warp and row.
+            constexpr int kUnit = 2 * NC;  // contiguous bytes of the slice
+            const uint32_t pcur = sbase + Lt::kPOff + (uint32_t)((k & 1) * Lt::kPBytes);
+            if (key < D) {
+                float o[NC];
+                const uint32_t o_t = tmem + lane_base + (uint32_t)(Lt::kOCol + col0);
+                if constexpr (D == 64) tmem_ld<NC>(o_t, o);
+#pragma unroll
+                for (int c = 0; c < NC; c += 16) {
+                    float lr[16];
+                    if constexpr (D == 128) {
+                        tmem_ld_two<16>(o_t + c, o_t + (Lt::kLCol - Lt::kOCol) + c, o + c, lr);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < 16; r += 4) {
+                            const float4 y = lds4(lr_sm + 4 * (c + r));
+                            lr[r] = y.x;
+                            lr[r + 1] = y.y;
+                            lr[r + 2] = y.z;
+                            lr[r + 3] = y.w;
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) o[c + r] *= inverse(lr[r]);
+                }
+                if (whole) {
+#pragma unroll
+                    for (int r = 0; r < NC; ++r)
+                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(
+                                         slice_at<N>(pcur, group, (r * D + key) * 2 / kUnit) +
+                                         key * 2 % kUnit),
+                                     "h"((uint16_t)pack_bf16(o[r], 0.f))
+                                     : "memory");
+                } else {
+                    float *ob = p.part_o + (slot * p.rows_max + col0) * D + key;
+#pragma unroll
+                    for (int r = 0; r < NC; ++r)
+                        if (r < rows_active) __stcg(ob + r * D, o[r]);
+                }
+            }
+            soft_sync(group);  // the row sums of all warps
+            if (key < NC && key < rows_active) {
+                const int r = key, qr = col0 + r;
+                const uint32_t red = red_sm + 4 * r;
+                const float lsum = (lds(red) + lds(red + 4 * N)) + (lds(red + 8 * N) + lds(red + 12 * N));
+                // m + log2(l), l's exponent apart: m and it may cancel
+                const float e = (float)((int)(__float_as_uint(lsum) >> 23) - 127);
+                const float f = __uint_as_float((__float_as_uint(lsum) & 0x7fffffu) | 0x3f800000u);
+                const float lse = lsum > 3.4e38f ? INFINITY
+                                  : lsum > 0.f
+                                      ? ((e - lds(nm_sm + 4 * r)) + __log2f(f)) * kLn2
+                                      : -INFINITY;
+                if (whole)
+                    p.lse[((size_t)w.b * p.Hq + (size_t)w.h * p.G + qr % p.G) * p.max_block +
+                          qr / p.G] = lse;
+                else
+                    p.part_lse[slot * p.rows_max + qr] = lse;
+            }
+            if (whole) {
+                for (int c = key; c < min(rows_active, NC) * (D / 8); c += 128) {
+                    const int r = c / (D / 8), x = c * 16;
+                    uint4 y;
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
+                                 : "r"(slice_at<N>(pcur, group, x / kUnit) + x % kUnit)
+                                 : "memory");
+                    const int qr = col0 + r;
+                    *reinterpret_cast<uint4 *>(
+                        p.out + (((size_t)w.b * p.max_block + qr / p.G) * p.Hq + (size_t)w.h * p.G +
+                                 qr % p.G) * D + (c % (D / 8)) * 8) = y;
+                }
+            }
+            soft_sync(group);  // the rows' values and the slice may be written again
+            if (whole) {  // rows past the block: 0 and lse -inf
+                const int act = p.G * w.T;
+                for (int idx = threadIdx.x; idx < (p.rows_max - act) * (D / 8);
+                     idx += kSoftWarps * 32) {
+                    const int r = act + idx / (D / 8), col = (idx % (D / 8)) * 8;
+                    const int ii = r / p.G, gg = r % p.G;
+                    *reinterpret_cast<uint4 *>(p.out + (((size_t)w.b * p.max_block + ii) *
+                                                             p.Hq +
+                                                         (size_t)w.h * p.G + gg) * D + col) =
+                        make_uint4(0u, 0u, 0u, 0u);
+                    if (col == 0)
+                        p.lse[((size_t)w.b * p.Hq + (size_t)w.h * p.G + gg) * p.max_block +
+                              ii] = -INFINITY;
+                }
+            }
+            fence_before();
+        }
+        ++k;
+        done += sg.tiles;
+        walk_segment(p, w, sg);
+        }
+    }
+    if (warp == kMmaWarp || warp == kSWarp) {
         // all MMAs this warp issued are complete before tensor memory is freed
         // (only a timed-out run can leave any in flight)
         const uint32_t drain = b_drain + (warp == kSWarp ? 8 : 0);
@@ -1277,581 +1501,27 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
         const unsigned long long t0 = globaltimer();
         while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < kWaitNs) {
         }
-    } else if (kQSplit && warp >= kConvWarp0) {
-        // ========================== query split (kQSplit) ========================
-        // Once a segment's bf16 query rows have landed, split them into their
-        // e4m3 parts for the S MMAs and record each row's e for the softmax
-        // warps (qsplit).  Query buffer b is loaded again only after the S of
-        // its segment and every softmax warp's read of e are done (qempty),
-        // so neither the parts nor e are overwritten early.
-        const int ct = threadIdx.x - kConvWarp0 * 32;
-        Walk wc = w0;
-        int qs = -1;
-        for (long long j = 0; j < ntiles; ++j) {
-            if (j == 0 || wc.t == 0) {
-                ++qs;
-                const int qb = qs & 1;
-                if (!wait(b_qfull + 8 * qb, (uint32_t)((qs >> 1) & 1), abort_flag, p.status))
-                    break;
-                const uint32_t q8 = sbase + Lt::kQ8Off + 2 * qb * Lt::kQ8Bytes;
-                split_q(sbase + Lt::kQOff + qb * Lt::kQBytes, q8, q8 + Lt::kQ8Bytes,
-                        qexp + qb * kRows, ct);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(b_qsplit + 8 * qb);
-            }
-            walk_next(p, wc);
-        }
-    } else if (Lt::kConv && warp >= kConvWarp0) {
-        // ============================ e4m3 -> bf16 ===============================
-        // Widen every prefix tile's e4m3 K (and V) into its ring slot once it
-        // has landed and the slot is free, then hand the tile to the S warp
-        // (cready).  A block tile's K (V) is bf16 already: for a ring operand
-        // one elected lane of the first conversion warp loads it into the slot
-        // with a copy that completes on cready itself.
-        const int ct = threadIdx.x - kConvWarp0 * 32;
-        Walk wc = w0;
-        bool ok = true;
-        for (long long j = 0; j < ntiles && ok; ++j) {
-            const int s = (int)(j % kStages);
-            const uint32_t cready = b_cready + 8 * (int)(j % kSlots);
-            ok = wait(b_full + 8 * s, (uint32_t)((j / kStages) & 1), abort_flag, p.status);
-            if (!ok) break;
-            if (wc.t == wc.nt - 1) {
-                if (KF8) ok = slot_free(b_kfree, j);
-                if (VF8) ok = ok && slot_free(b_vfree, j);
-                if (!ok) break;
-                if (warp == kConvWarp0) {
-                    if (elect_one()) {
-                        mbar_arrive_expect_tx(cready, ((KF8 ? 1 : 0) + (VF8 ? 1 : 0)) *
-                                                          Lt::kTileBytes);
-#pragma unroll
-                        for (int dp = 0; dp < Lt::kPanels; ++dp) {
-                            if (KF8)
-                                tma_4d(k_src(s, j) + dp * 8192, &tm_kb, cready, dp * 64, wc.h, 0,
-                                       wc.b);
-                            if (VF8)
-                                tma_4d(v_src(s, j) + dp * 8192, &tm_vb, cready, dp * 64, wc.h, 0,
-                                       wc.b);
-                        }
-                    }
-                    drain_copy = j;
-                } else if (lane == 0) {
-                    mbar_arrive(cready);
-                }
-                __syncwarp();
-                walk_next(p, wc);
-                continue;
-            }
-            if (KF8) {
-                ok = slot_free(b_kfree, j);
-                if (!ok) break;
-                widen_tile<D>(sbase + s * Lt::kStageBytes, k_src(s, j), ct);
-            }
-            if (VF8) {
-                ok = slot_free(b_vfree, j);
-                if (!ok) break;
-                widen_tile<D>(sbase + s * Lt::kStageBytes + Lt::kKBytes, v_src(s, j), ct);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(cready);
-            walk_next(p, wc);
-        }
-    } else {
-        // ================================ softmax ================================
-        // thread (warp, lane) handles row 16 warp + lane % 16, keys of its half
-        // (lane / 16) of each tile; the epilogue's O rows are read by lanes < 16
-        const int row = warp * 16 + (lane & 15);
-        // (REP) MMA row c 64 / NC + r holds copy c of query row r: warp w
-        // holds rows of copy cp = w / (4 / NC)
-        constexpr int kRowsPerCopy = kRows / NC;
-        const int cp = REP ? warp / (4 / NC) : 0;
-        const int qrow = REP ? row - cp * kRowsPerCopy : row;
-        const int half = lane >> 4;
-        // scores a thread takes per tile, and the first of them
-        constexpr int kVals = 32 / NC;
-        const int key0 = cp * (kTileKeys / NC) + kVals * half;
-        const bool owner = lane < 16;
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-        Walk ws = w0;
-        // l_sum: sum of the fp32 weights 2^(s - m), for the lse.  The sum of
-        // the same weights as rounded to bf16 for the P V product, used for
-        // the normalisation so that O / l is an exact convex combination of
-        // the values (the rounding of P then moves the output by a fraction
-        // of the values' spread around it, not of the values themselves), is
-        // accumulated by the tensor core next to O (P times a ones column,
-        // fp32), which takes its tree of adds off the softmax warps.
-        float m_ref = -INFINITY, l_sum = 0.f;
-        int rows_active = 0, irow = 0;
-        long long seg_first = lo;
-        // (kQSplit) scale of the prefix tiles' scores: S holds 2^e q.k for this row
-        float row_scale = p.scale_log2;
-        int qs = -1;
-        for (long long k = 0; k < ntiles; ++k) {
-            const bool first = (k == 0) || (ws.t == 0);
-            const bool block_tile = ws.t == ws.nt - 1;
-            const bool last = block_tile || (k + 1 == ntiles);
-            if (first) {
-                m_ref = -INFINITY;
-                l_sum = 0.f;
-                rows_active = p.G * ws.T;
-                irow = qrow / p.G;
-                seg_first = lo + k;
-                if (kQSplit) {
-                    ++qs;
-                    const int qb = qs & 1;
-                    wait(b_qsplit + 8 * qb, (uint32_t)((qs >> 1) & 1), abort_flag, p.status);
-                    const int e = qexp[qb * kRows + row];
-                    row_scale = p.scale_log2 * __uint_as_float((uint32_t)(127 - e) << 23);
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(b_qempty + 8 * qb);
-                }
-            }
-            const int nvalid = block_tile ? ws.T : min(kTileKeys, ws.P - ws.t * kTileKeys);
-            const int s = (int)(k % kStages);
-            // ---- scores of tile k ----
-            const bool ok_s = wait(b_sready + 8 * (int)(k % kSBufs),
-                                   (uint32_t)((k / kSBufs) & 1), abort_flag, p.status);
-            fence_after();
-            const uint32_t s_addr = tmem + lane_base + (uint32_t)((k % kSBufs) * kTileKeys) +
-                                    (uint32_t)(cp * (kTileKeys / NC));
-            const bool valid_row = qrow < rows_active && ok_s;
-            // keys j < lim are visible to this row; a full prefix tile needs no
-            // mask (rows of other lanes are computed but never stored)
-            const int lim = !valid_row ? 0 : (block_tile ? min(nvalid, irow + 1) : nvalid);
-            const bool full_tile = !block_tile && nvalid == kTileKeys;
-            const float scale = kQSplit && !block_tile ? row_scale : p.scale_log2;
-            // The thread's 32 scores in registers (masked keys -> -inf); the
-            // row's tile max decides the reference first: the segment's first
-            // tile sets it, a later tile moves it (rescaling O and l) only when
-            // its max is beyond the reference by more than 2^8.
-            float v[kVals];
-            if constexpr (kVals == 8)
-                tmem_ld_half8(s_addr, v);
-            else if constexpr (kVals == 16)
-                tmem_ld_half16(s_addr, v);
-            else
-                tmem_ld_half32(s_addr, v);
-            // the scores are in registers: S buffer k % kSBufs may take tile k + kSBufs
-            fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_sfree + 8 * (int)(k % kSBufs));
-            if (!full_tile) {
-#pragma unroll
-                for (int j = 0; j < kVals; j += 2) {
-                    float a, b;
-                    mul2(a, b, v[j], v[j + 1], scale, scale);
-                    v[j] = key0 + j < lim ? a : -INFINITY;
-                    v[j + 1] = key0 + j + 1 < lim ? b : -INFINITY;
-                }
-            }
-            float mt;
-            if constexpr (kVals == 8) {
-                const float m = max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]), fmaxf(v[6], v[7]));
-                mt = full_tile ? m * scale : m;
-            } else if constexpr (kVals == 16) {  // 16 -> 6 -> 2 -> 1
-                const float m = fmaxf(max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]),
-                                           max3(v[6], v[7], v[8])),
-                                      max3(max3(v[9], v[10], v[11]), max3(v[12], v[13], v[14]), v[15]));
-                mt = full_tile ? m * scale : m;
-            } else {  // three-input maxima: 32 -> 11 -> 4 -> 1
-                float m11[11];
-#pragma unroll
-                for (int j = 0; j < 10; ++j) m11[j] = max3(v[3 * j], v[3 * j + 1], v[3 * j + 2]);
-                m11[10] = fmaxf(v[30], v[31]);
-                const float m = fmaxf(max3(max3(m11[0], m11[1], m11[2]), max3(m11[3], m11[4], m11[5]),
-                                           max3(m11[6], m11[7], m11[8])),
-                                      fmaxf(m11[9], m11[10]));
-                mt = full_tile ? m * scale : m;
-            }
-            mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 16));
-            if (first) {
-                m_ref = mt;
-            } else {
-                const bool jump = valid_row && mt > m_ref + kRescaleLog2;
-                if (__any_sync(kFull, jump)) {
-                    // O is stable once P V of tile k-1 is done
-                    wait(b_pvdone + 8 * (int)((k - 1) & 1), (uint32_t)(((k - 1) >> 1) & 1),
-                         abort_flag, p.status);
-                    fence_after();
-                    const float alpha = jump ? ex2(m_ref - mt) : 1.f;  // m_ref -inf gives 0
-                    if (jump) {
-                        m_ref = mt;
-                        l_sum *= alpha;
-                    }
-                    // O and, in the next 32 columns, the rounded row sum
-#pragma unroll 1
-                    for (int c = 0; c < D + 32; c += 32) {
-                        float o[32];
-                        const uint32_t ta = tmem + lane_base + (uint32_t)(kSBufs * kTileKeys + c);
-                        tmem_ld32(ta, o);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) o[j] *= alpha;
-                        tmem_st32(ta, o);
-                    }
-                }
-            }
-            // P = 2^(s - m) as bf16 into the swizzled P buffer (32 keys = 4
-            // chunks): all exponentials first, then the packs (measured faster
-            // than one loop that does both per pair); their tree sum for l
-            // comes after P has been handed on
-            const float mu = m_ref == -INFINITY ? 0.f : m_ref;
-            if (full_tile) {
-#pragma unroll
-                for (int j = 0; j < kVals; j += 2)
-                    fma2(v[j], v[j + 1], v[j], v[j + 1], scale, scale, -mu, -mu);
-            } else {
-#pragma unroll
-                for (int j = 0; j < kVals; j += 2) add2(v[j], v[j + 1], v[j], v[j + 1], -mu, -mu);
-            }
-#pragma unroll
-            for (int j = 0; j < kVals; ++j) v[j] = ex2(v[j]);
-            uint32_t w[kVals / 2];
-#pragma unroll
-            for (int e = 0; e < kVals / 2; ++e) w[e] = pack_bf16(v[2 * e], v[2 * e + 1]);
-            // P buffer (k & 1) is free once P V of tile k-2, its last reader, is done
-            // (pvdone[k & 1] completes once per P V of tiles with that parity)
-            if (k >= 2) wait(b_pvdone + 8 * (int)(k & 1), (uint32_t)(((k - 2) >> 1) & 1), abort_flag,
-                             p.status);
-            fence_after();
-            const uint32_t pbuf = sbase + Lt::kPOff + (uint32_t)((k & 1) * Lt::kPBytes);
-#pragma unroll
-            for (int q4 = 0; q4 < kVals / 8; ++q4)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                                 p_chunk_addr(pbuf, row, key0 / 8 + q4)),
-                             "r"(w[4 * q4]), "r"(w[4 * q4 + 1]), "r"(w[4 * q4 + 2]),
-                             "r"(w[4 * q4 + 3])
-                             : "memory");
-            // keys past the end of the tile may hold anything: zero their V rows
-            if (nvalid < kTileKeys) {
-                const uint32_t vt = v_src(s, k);
-                const int nzero = (kTileKeys - nvalid) * 8 * Lt::kPanels;  // 16-byte chunks
-                for (int i = threadIdx.x; i < nzero; i += kSoftWarps * 32) {
-                    const int panel = i / ((kTileKeys - nvalid) * 8);
-                    const int rem = i % ((kTileKeys - nvalid) * 8);
-                    const int key = nvalid + rem / 8, chunk = rem % 8;
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
-                                     vt + panel * 8192 + key * 128 + (chunk << 4)),
-                                 "r"(0u)
-                                 : "memory");
-                }
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_pready + 8 * (int)(k & 1));
-            if constexpr (kVals == 8) {
-                l_sum += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
-            } else if constexpr (kVals == 16) {
-                float a0, a1, b0, b1;
-                add2(a0, a1, v[0], v[1], v[8], v[9]);
-                add2(b0, b1, v[2], v[3], v[10], v[11]);
-                float c0, c1, d0, d1;
-                add2(c0, c1, v[4], v[5], v[12], v[13]);
-                add2(d0, d1, v[6], v[7], v[14], v[15]);
-                add2(a0, a1, a0, a1, c0, c1);
-                add2(b0, b1, b0, b1, d0, d1);
-                add2(a0, a1, a0, a1, b0, b1);
-                l_sum += a0 + a1;
-            } else {  // the row sum is needed only for l: after P has been handed on
-                // (packed adds, in the order of the tree t[j] += t[j + w])
-                float t[16];
-#pragma unroll
-                for (int j = 0; j < 16; j += 2)
-                    add2(t[j], t[j + 1], v[j], v[j + 1], v[j + 16], v[j + 17]);
-#pragma unroll
-                for (int wd = 8; wd > 1; wd >>= 1)
-#pragma unroll
-                    for (int j = 0; j < wd; j += 2)
-                        add2(t[j], t[j + 1], t[j], t[j + 1], t[j + wd], t[j + wd + 1]);
-                l_sum += t[0] + t[1];
-            }
-
-            // ---- end of segment: O / l and lse ----
-            if (last) {
-                wait(b_pvdone + 8 * (int)(k & 1), (uint32_t)((k >> 1) & 1), abort_flag, p.status);
-                fence_after();
-                const long long pair_first = lo + k - ws.t;
-                const bool whole = (seg_first == pair_first) && block_tile;
-                const int pair = ws.b * p.Hkv + ws.h;
-                const size_t slot = (size_t)pair + blockIdx.x;
-                const bool write = qrow < rows_active;
-                // the row's sums: this thread's half plus its partner's; the
-                // rounded one from the tensor core (column 0 of the row-sum
-                // accumulator in the low half, column 1, zero, in the high one)
-                const float l_row = l_sum + __shfl_xor_sync(kFull, l_sum, 16);
-                float l_rnd;
-                {
-                    uint32_t r;
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.16x32bx2.x1.b32 {%0}, [%1], 1;\n"
-                        "tcgen05.wait::ld.sync.aligned;"
-                        : "=r"(r)
-                        : "r"(tmem + lane_base + (uint32_t)(kSBufs * kTileKeys + D))
-                        : "memory");
-                    l_rnd = __uint_as_float(r);
-                }
-                const float l_row_rnd = l_rnd + __shfl_xor_sync(kFull, l_rnd, 16);
-                const int gq = qrow % p.G;
-                // this thread's columns: [64 g + 32 half, +32) for each 64-column group g
-                float v[D / 2];
-                tmem_ld_orow<D>(tmem + lane_base + (uint32_t)(kSBufs * kTileKeys), v);
-                if constexpr (REP && Lt::kCompactXch) {
-                    // The NC copies of each row through shared memory: the
-                    // groups of its O row (not normalised) that the other
-                    // copies combine, and its (m, l, rounded l); then thread
-                    // (copy cp, row r, half) combines group cp of half `half`
-                    // of query row r by log-sum-exp over the copies.
-                    constexpr int kG = D / 2 / NC;  // values per group
-                    constexpr int kXS = Lt::kXchStride;
-                    float *xo = reinterpret_cast<float *>(sm + Lt::kXchOff);
-                    float *xm = xo + 2 * kRows * kXS;
-                    float *dst = xo + (half * kRows + row) * kXS;
-#pragma unroll
-                    for (int g = 0; g < NC; ++g) {
-                        if (g == cp) continue;
-                        const int slot = g < cp ? g : g - 1;
-#pragma unroll
-                        for (int j = 0; j < kG; j += 4)
-                            *reinterpret_cast<float4 *>(dst + slot * kG + j) =
-                                make_float4(v[g * kG + j], v[g * kG + j + 1], v[g * kG + j + 2],
-                                            v[g * kG + j + 3]);
-                    }
-                    if (half == 0)
-                        *reinterpret_cast<float4 *>(xm + row * 4) =
-                            make_float4(m_ref, l_row, l_row_rnd, 0.f);
-                    // this thread's own group, selected without a dynamic register index
-                    constexpr int kDims = kG;
-                    float own[kG];
-#pragma unroll
-                    for (int j = 0; j < kG; ++j) own[j] = v[j];
-#pragma unroll
-                    for (int g = 1; g < NC; ++g)
-                        if (cp == g)
-#pragma unroll
-                            for (int j = 0; j < kG; ++j) own[j] = v[g * kG + j];
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    // group cp's dims: values [0, 32) of a half are dims 32 half + i,
-                    // values [32, 64) dims 64 + 32 half + i - 32
-                    const int i0 = cp * kG;
-                    const int d0 = i0 < 32 ? 32 * half + i0 : 64 + 32 * half + (i0 - 32);
-                    float4 ml[NC];
-                    float M = -INFINITY;
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        ml[c] = *reinterpret_cast<const float4 *>(xm + (c * kRowsPerCopy + qrow) * 4);
-                        M = fmaxf(M, ml[c].x);
-                    }
-                    float L = 0.f, Lr = 0.f, o[kDims];
-#pragma unroll
-                    for (int j = 0; j < kDims; ++j) o[j] = 0.f;
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        // a copy that saw no visible key has m = -inf and weight 0
-                        const float sc = ml[c].x == -INFINITY ? 0.f : ex2(ml[c].x - M);
-                        L += sc * ml[c].y;
-                        Lr += sc * ml[c].z;
-                        if (c == cp) {
-#pragma unroll
-                            for (int j = 0; j < kDims; ++j) o[j] += sc * own[j];
-                        } else {
-                            const float *src = xo + (half * kRows + c * kRowsPerCopy + qrow) * kXS +
-                                               (cp < c ? cp : cp - 1) * kG;
-#pragma unroll
-                            for (int j = 0; j < kDims; j += 4) {
-                                const float4 x = *reinterpret_cast<const float4 *>(src + j);
-                                o[j] += sc * x.x;
-                                o[j + 1] += sc * x.y;
-                                o[j + 2] += sc * x.z;
-                                o[j + 3] += sc * x.w;
-                            }
-                        }
-                    }
-                    const float inv = Lr > 0.f ? 1.f / Lr : 0.f;
-                    const float lse = L > 0.f ? (M + __log2f(L)) * kLn2 : -INFINITY;
-                    if (write) {
-                        if (whole) {
-                            uint16_t *orow = p.out + (((size_t)ws.b * p.max_block + irow) * p.Hq +
-                                                      (size_t)ws.h * p.G + gq) * D + d0;
-#pragma unroll
-                            for (int j = 0; j < kDims; j += 8)
-                                *reinterpret_cast<uint4 *>(orow + j) =
-                                    make_uint4(pack_bf16(o[j] * inv, o[j + 1] * inv),
-                                               pack_bf16(o[j + 2] * inv, o[j + 3] * inv),
-                                               pack_bf16(o[j + 4] * inv, o[j + 5] * inv),
-                                               pack_bf16(o[j + 6] * inv, o[j + 7] * inv));
-                        } else {
-                            float *prow = p.part_o + (slot * p.rows_max + qrow) * D + d0;
-#pragma unroll
-                            for (int j = 0; j < kDims; j += 4)
-                                *reinterpret_cast<float4 *>(prow + j) =
-                                    make_float4(o[j] * inv, o[j + 1] * inv, o[j + 2] * inv,
-                                                o[j + 3] * inv);
-                        }
-                        if (cp == 0 && half == 0) {
-                            if (whole)
-                                p.lse[((size_t)ws.b * p.Hq + (size_t)ws.h * p.G + gq) *
-                                          p.max_block +
-                                      irow] = lse;
-                            else
-                                p.part_lse[slot * p.rows_max + qrow] = lse;
-                        }
-                    }
-                    // the exchange area is free again once every thread has read it
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                } else if constexpr (REP) {
-                    // The NC copies of each row through shared memory: every
-                    // copy's O row (not normalised) and its (m, l, rounded l);
-                    // then thread (copy cp, row r, half) combines kDims dims of
-                    // query row r, from kDims (2 cp + half), by log-sum-exp
-                    // over the copies.
-                    constexpr int kDims = kRowsPerCopy * D / 128;
-                    float *xo = reinterpret_cast<float *>(sm + Lt::kXchOff);
-                    float *xm = xo + kRows * Lt::kXchStride;
-                    float *dst = xo + row * Lt::kXchStride + 32 * half;
-#pragma unroll
-                    for (int g = 0; g < D / 64; ++g)
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4)
-                            *reinterpret_cast<float4 *>(dst + 64 * g + j) =
-                                make_float4(v[32 * g + j], v[32 * g + j + 1], v[32 * g + j + 2],
-                                            v[32 * g + j + 3]);
-                    if (half == 0)
-                        *reinterpret_cast<float4 *>(xm + row * 4) =
-                            make_float4(m_ref, l_row, l_row_rnd, 0.f);
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    const int d0 = kDims * (2 * cp + half);
-                    float4 ml[NC];
-                    float M = -INFINITY;
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        ml[c] = *reinterpret_cast<const float4 *>(xm + (c * kRowsPerCopy + qrow) * 4);
-                        M = fmaxf(M, ml[c].x);
-                    }
-                    float L = 0.f, Lr = 0.f, o[kDims];
-#pragma unroll
-                    for (int j = 0; j < kDims; ++j) o[j] = 0.f;
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        // a copy that saw no visible key has m = -inf and weight 0
-                        const float sc = ml[c].x == -INFINITY ? 0.f : ex2(ml[c].x - M);
-                        L += sc * ml[c].y;
-                        Lr += sc * ml[c].z;
-                        const float *src = xo + (c * kRowsPerCopy + qrow) * Lt::kXchStride + d0;
-#pragma unroll
-                        for (int j = 0; j < kDims; j += 4) {
-                            const float4 x = *reinterpret_cast<const float4 *>(src + j);
-                            o[j] += sc * x.x;
-                            o[j + 1] += sc * x.y;
-                            o[j + 2] += sc * x.z;
-                            o[j + 3] += sc * x.w;
-                        }
-                    }
-                    const float inv = Lr > 0.f ? 1.f / Lr : 0.f;
-                    const float lse = L > 0.f ? (M + __log2f(L)) * kLn2 : -INFINITY;
-                    if (write) {
-                        if (whole) {
-                            uint16_t *orow = p.out + (((size_t)ws.b * p.max_block + irow) * p.Hq +
-                                                      (size_t)ws.h * p.G + gq) * D + d0;
-#pragma unroll
-                            for (int j = 0; j < kDims; j += 8)
-                                *reinterpret_cast<uint4 *>(orow + j) =
-                                    make_uint4(pack_bf16(o[j] * inv, o[j + 1] * inv),
-                                               pack_bf16(o[j + 2] * inv, o[j + 3] * inv),
-                                               pack_bf16(o[j + 4] * inv, o[j + 5] * inv),
-                                               pack_bf16(o[j + 6] * inv, o[j + 7] * inv));
-                        } else {
-                            float *prow = p.part_o + (slot * p.rows_max + qrow) * D + d0;
-#pragma unroll
-                            for (int j = 0; j < kDims; j += 4)
-                                *reinterpret_cast<float4 *>(prow + j) =
-                                    make_float4(o[j] * inv, o[j + 1] * inv, o[j + 2] * inv,
-                                                o[j + 3] * inv);
-                        }
-                        if (cp == 0 && half == 0) {
-                            if (whole)
-                                p.lse[((size_t)ws.b * p.Hq + (size_t)ws.h * p.G + gq) *
-                                          p.max_block +
-                                      irow] = lse;
-                            else
-                                p.part_lse[slot * p.rows_max + qrow] = lse;
-                        }
-                    }
-                    // the exchange area is free again once every thread has read it
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                } else {
-                const float inv = l_row_rnd > 0.f ? 1.f / l_row_rnd : 0.f;
-                const float lse = l_row > 0.f ? (m_ref + __log2f(l_row)) * kLn2 : -INFINITY;
-                if (write) {
-                    uint16_t *orow = p.out + (((size_t)ws.b * p.max_block + irow) * p.Hq +
-                                              (size_t)ws.h * p.G + gq) * D + 32 * half;
-                    float *prow = p.part_o + (slot * p.rows_max + row) * D + 32 * half;
-#pragma unroll
-                    for (int g = 0; g < D / 64; ++g) {
-                        const float *x = v + 32 * g;
-                        if (whole) {
-#pragma unroll
-                            for (int j = 0; j < 32; j += 8)
-                                *reinterpret_cast<uint4 *>(orow + 64 * g + j) =
-                                    make_uint4(pack_bf16(x[j] * inv, x[j + 1] * inv),
-                                               pack_bf16(x[j + 2] * inv, x[j + 3] * inv),
-                                               pack_bf16(x[j + 4] * inv, x[j + 5] * inv),
-                                               pack_bf16(x[j + 6] * inv, x[j + 7] * inv));
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 32; j += 4)
-                                *reinterpret_cast<float4 *>(prow + 64 * g + j) =
-                                    make_float4(x[j] * inv, x[j + 1] * inv, x[j + 2] * inv,
-                                                x[j + 3] * inv);
-                        }
-                    }
-                }
-                if (write && owner) {
-                    if (whole)
-                        p.lse[((size_t)ws.b * p.Hq + (size_t)ws.h * p.G + gq) * p.max_block +
-                              irow] = lse;
-                    else
-                        p.part_lse[slot * p.rows_max + row] = lse;
-                }
-                }  // REP
-                if (whole) {  // rows past the block: 0 and lse -inf
-                    for (int idx = threadIdx.x; idx < (p.rows_max - rows_active) * (D / 8);
-                         idx += kSoftWarps * 32) {
-                        const int r = rows_active + idx / (D / 8), col = (idx % (D / 8)) * 8;
-                        const int ii = r / p.G, gg = r % p.G;
-                        *reinterpret_cast<uint4 *>(p.out + (((size_t)ws.b * p.max_block + ii) *
-                                                                 p.Hq +
-                                                             (size_t)ws.h * p.G + gg) * D + col) =
-                            make_uint4(0u, 0u, 0u, 0u);
-                        if (col == 0)
-                            p.lse[((size_t)ws.b * p.Hq + (size_t)ws.h * p.G + gg) * p.max_block +
-                                  ii] = -INFINITY;
-                    }
-                }
-                fence_before();
-            }
-            walk_next(p, ws);
-        }
     }
-    // every MMA was waited on by the control lane and the softmax warps
+    // every MMA was waited on by its issuing warp and the softmax warps
     fence_before();
     __syncthreads();
     fence_after();
-    if (*abort_flag) {  // a wait gave up: copies still in flight land before exit
+    if (lds(abort_flag) != 0.f) {  // a wait gave up: copies still in flight land before exit
         if (warp == kProducerWarp && elect_one()) {
-            for (long long j = drain_tiles - 1; j >= 0 && j >= drain_tiles - kStages; --j)
-                drain_wait(b_full + 8 * (int)(j % kStages), (uint32_t)((j / kStages) & 1));
-            for (int q = drain_qseg; q >= 0 && q >= drain_qseg - 1; --q)
+            for (int s = loads - 1; s >= 0 && s >= loads - VS; --s)
+                drain_wait(b_vfull + 8 * (s % VS), (uint32_t)((s / VS) & 1));
+            for (int q = qseg; q >= 0 && q >= qseg - 1; --q)
                 drain_wait(b_qfull + 8 * (q & 1), (uint32_t)((q >> 1) & 1));
         }
-        if (Lt::kConv && warp == kConvWarp0 && lane == 0 && drain_copy >= 0)
-            drain_wait(b_cready + 8 * (int)(drain_copy % kSlots),
-                       (uint32_t)((drain_copy / kSlots) & 1));
+        if (warp == kSWarp && elect_one())
+            for (int s = kloads - 1; s >= 0 && s >= kloads - KS; --s)
+                drain_wait(b_kfull + 8 * (s % KS), (uint32_t)((s / KS) & 1));
+        if (VF8 && warp == kConvWarp0 && lane == 0 && drain_copy >= 0)
+            drain_wait(b_wready + 8 * (drain_copy % WS), (uint32_t)((drain_copy / WS) & 1));
     }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "n"(kTmemCols));
+                     "n"(Lt::kTmemCols));
 }
 
 }  // namespace
@@ -2021,8 +1691,14 @@ cudaError_t merge_occupancy(int dev, int occ[kMergeVariants]) {
         reinterpret_cast<const void *>(merge_kernel<D, 2, 1>),
         reinterpret_cast<const void *>(merge_kernel<D, 2, 2>)};
     for (int v = 0; v < kMergeVariants; ++v) {
-        const cudaError_t e =
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[v], fns[v], kMergeWarps * 32, 0);
+        // few pairs: the shared-memory split of the attention kernel that the merge runs
+        // beside; many rows to merge read faster with the default's larger L1
+        cudaError_t e = cudaSuccess;
+        if (kMergeSegs[v] > 2)
+            e = cudaFuncSetAttribute(fns[v], cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[v], fns[v], kMergeWarps * 32, 0);
         if (e != cudaSuccess) return e;
         occ[v] = std::max(occ[v], 1);
     }
@@ -2034,19 +1710,24 @@ cudaError_t merge_occupancy(int dev, int occ[kMergeVariants]) {
     return cudaSuccess;
 }
 
-template <int D, bool KF8, bool VF8, int NC = 1>
-cudaError_t launch_d(const AttnParams &p, const CUtensorMap &tk, const CUtensorMap &tv,
+template <int D, bool KF8, bool VF8, int N>
+cudaError_t launch_n(const AttnParams &p, const CUtensorMap &tk, const CUtensorMap &tk2,
+                     const CUtensorMap &tv,
                      const CUtensorMap &tkb, const CUtensorMap &tvb, const CUtensorMap &tq,
                      cudaStream_t stream) {
-    using Lt = Layout<D, KF8, VF8, NC>;
+    using Lt = Layout<D, KF8, VF8, N>;
     constexpr int smem = Lt::kBytes;
     static std::atomic<bool> configured[64];  // the smem opt-in, once per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(attn_kernel<D, KF8, VF8, NC>,
+        e = cudaFuncSetAttribute(attn_kernel<D, KF8, VF8, N>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(attn_kernel<D, KF8, VF8, N>,
+                                 cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         if (dev < 64) configured[dev].store(true, std::memory_order_release);
     }
@@ -2060,8 +1741,22 @@ cudaError_t launch_d(const AttnParams &p, const CUtensorMap &tk, const CUtensorM
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, attn_kernel<D, KF8, VF8, NC>, tk, tv, tkb, tvb, tq, p);
+    return cudaLaunchKernelEx(&cfg, attn_kernel<D, KF8, VF8, N>, tk, tk2, tv, tkb, tvb, tq, p);
+}
+
+// The merge, a programmatic dependent of either attention kernel.
+template <int D>
+cudaError_t launch_merge(const AttnParams &p, cudaStream_t stream) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     // The merge variant with the fewest estimated sequential steps: waves of
     // resident merge CTAs (at least one) times L2 round trips per row (at
     // least one), for a pair's average segment count 1 + C / (B Hkv).
@@ -2093,6 +1788,35 @@ cudaError_t launch_d(const AttnParams &p, const CUtensorMap &tk, const CUtensorM
     return cudaLaunchKernelEx(&cfg, merge_kernel<D, 2, 2>, p);
 }
 
+// The MMAs' query columns: the pair's G * max_block rows rounded up to 16, 32 or 64.
+template <int D, bool KF8, bool VF8>
+cudaError_t launch_d(const AttnParams &p, const CUtensorMap &tk, const CUtensorMap &tk2,
+                     const CUtensorMap &tv,
+                     const CUtensorMap &tkb, const CUtensorMap &tvb, const CUtensorMap &tq,
+                     cudaStream_t stream) {
+    if (p.rows_max <= 16) return launch_n<D, KF8, VF8, 16>(p, tk, tk2, tv, tkb, tvb, tq, stream);
+    if (p.rows_max <= 32) return launch_n<D, KF8, VF8, 32>(p, tk, tk2, tv, tkb, tvb, tq, stream);
+    return launch_n<D, KF8, VF8, 64>(p, tk, tk2, tv, tkb, tvb, tq, stream);
+}
+
+cudaError_t launch_attn(const AttnParams &p, int head_dim, bool keys_e4m3, bool values_e4m3,
+                        const CUtensorMap &tk, const CUtensorMap &tk2, const CUtensorMap &tv,
+                        const CUtensorMap &tkb, const CUtensorMap &tvb, const CUtensorMap &tq,
+                        cudaStream_t stream) {
+#define DAS_LAUNCH(D, K8, V8) launch_d<D, K8, V8>(p, tk, tk2, tv, tkb, tvb, tq, stream)
+    if (head_dim == 128) {
+        if (keys_e4m3)
+            return values_e4m3 ? DAS_LAUNCH(128, true, true) : DAS_LAUNCH(128, true, false);
+        return values_e4m3 ? DAS_LAUNCH(128, false, true) : DAS_LAUNCH(128, false, false);
+    }
+    if (head_dim == 64) {
+        if (keys_e4m3) return values_e4m3 ? DAS_LAUNCH(64, true, true) : DAS_LAUNCH(64, true, false);
+        return values_e4m3 ? DAS_LAUNCH(64, false, true) : DAS_LAUNCH(64, false, false);
+    }
+#undef DAS_LAUNCH
+    return cudaErrorInvalidValue;
+}
+
 }  // namespace tc
 
 int attn_grid_size(int device) {
@@ -2106,6 +1830,35 @@ int attn_grid_size(int device) {
         return 0;
     if (device >= 0 && device < 64) sms_of[device].store(sms, std::memory_order_relaxed);
     return sms;
+}
+
+// Whether a call takes the kernel for short ranges (das_rows.cu).  The transposed
+// kernel costs less per tile and 0.3 to 1.5 us more per segment, so it is taken
+// where the average segment, tiles / (pairs + CTAs), is long enough.  The prefix
+// lengths are the device's; the capacity bounds them.  Measured, time of the
+// short-range kernel over the transposed one's at that many tiles a segment:
+//   bf16 D = 128, N = 16: 1.6 0.95, 3.8 1.03, 5.7 1.01, 12 1.06;  N = 32 and 64: 3.2 0.96,
+//     5.7 0.96, 9.8 1.00, 10 1.03
+//   bf16 D = 64, N = 16: 1.6 1.01, 5.7 1.09, 12 1.38;  wider: 3.2 0.88, 5.7 0.95, 9.8 1.00
+//   e4m3 keys D = 128, N = 16: 1.6 1.09, 5.7 1.05, 18 1.14;  wider: 3.2 0.93, 5.7 0.99, 9.8 1.02
+//   e4m3 keys and values D = 128, N = 16: 1.6 1.01, 5.7 1.20, but over 256 pairs 3.8 0.91,
+//     6 0.92, over 512 12 1.20;  wider: 5.1 0.92, 9.8 1.04, 10 0.91 (256 pairs)
+//   the same at D = 64, N = 16: 5.7 0.95, 12 1.11, 18 1.31;  wider: 9.8 0.93, 10 0.88
+bool attn_short_ranges(int device, int batch, int kv_heads, int capacity, int head_dim,
+                       int rows_max, bool keys_e4m3, bool values_e4m3) {
+    const long long pairs = (long long)batch * kv_heads, C = attn_grid_size(device);
+    const long long tiles = pairs * ((capacity + kTileKeys - 1) / kTileKeys + 1);
+    const bool wide = rows_max > 16;
+    int need;
+    if (!keys_e4m3 && !values_e4m3)
+        need = wide ? 9 : 3;
+    else if (!values_e4m3 && head_dim == 128)
+        need = wide ? 9 : 1;
+    else if (head_dim == 128)
+        need = wide ? 11 : pairs > C ? 12 : 4;
+    else
+        need = wide ? 16 : pairs > C ? 12 : 9;
+    return tiles < need * (pairs + C);
 }
 
 namespace {
@@ -2133,34 +1886,20 @@ void attn_workspace_layout(void *workspace, int batch, int kv_heads, int rows_ma
     p.part_lse = reinterpret_cast<float *>(ws + off);
 }
 
-cudaError_t attn_launch(const AttnParams &p, int head_dim, bool keys_e4m3, bool values_e4m3,
-                        const CUtensorMap &tm_k, const CUtensorMap &tm_v,
+cudaError_t attn_launch(AttnParams p, int head_dim, bool keys_e4m3, bool values_e4m3,
+                        const CUtensorMap &tm_k, const CUtensorMap &tm_k2, const CUtensorMap &tm_v,
                         const CUtensorMap &tm_kb, const CUtensorMap &tm_vb,
                         const CUtensorMap &tm_q, cudaStream_t stream) {
-#define DAS_LAUNCH(D, K8, V8) tc::launch_d<D, K8, V8>(p, tm_k, tm_v, tm_kb, tm_vb, tm_q, stream)
-    if (head_dim == 128) {
-        if (keys_e4m3) {
-            if (values_e4m3) return DAS_LAUNCH(128, true, true);
-            if (p.rows_max <= 16)
-                return tc::launch_d<128, true, false, 4>(p, tm_k, tm_v, tm_kb, tm_vb, tm_q, stream);
-            if (p.rows_max <= 32)
-                return tc::launch_d<128, true, false, 2>(p, tm_k, tm_v, tm_kb, tm_vb, tm_q, stream);
-            return DAS_LAUNCH(128, true, false);
-        }
-        if (values_e4m3) return DAS_LAUNCH(128, false, true);
-        // at most 16 (32) rows per pair: four (two) copies of the rows (see attn_kernel)
-        if (p.rows_max <= 16)
-            return tc::launch_d<128, false, false, 4>(p, tm_k, tm_v, tm_kb, tm_vb, tm_q, stream);
-        if (p.rows_max <= 32)
-            return tc::launch_d<128, false, false, 2>(p, tm_k, tm_v, tm_kb, tm_vb, tm_q, stream);
-        return DAS_LAUNCH(128, false, false);
-    }
-    if (head_dim == 64) {
-        if (keys_e4m3) return values_e4m3 ? DAS_LAUNCH(64, true, true) : DAS_LAUNCH(64, true, false);
-        return values_e4m3 ? DAS_LAUNCH(64, false, true) : DAS_LAUNCH(64, false, false);
-    }
-#undef DAS_LAUNCH
-    return cudaErrorInvalidValue;
+    const int tile_bytes = kTileKeys * head_dim * ((keys_e4m3 ? 1 : 2) + (values_e4m3 ? 1 : 2));
+    p.block_weight = p.short_ranges ? 3 : tc::kBlockBytes / tile_bytes;
+    cudaError_t e;
+    if (p.short_ranges)
+        e = rows_launch(p, head_dim, keys_e4m3, values_e4m3, tm_k, tm_v, tm_kb, tm_vb, tm_q, stream);
+    else
+        e = tc::launch_attn(p, head_dim, keys_e4m3, values_e4m3, tm_k, tm_k2, tm_v, tm_kb, tm_vb, tm_q,
+                            stream);
+    if (e != cudaSuccess) return e;
+    return head_dim == 128 ? tc::launch_merge<128>(p, stream) : tc::launch_merge<64>(p, stream);
 }
 
 }  // namespace das

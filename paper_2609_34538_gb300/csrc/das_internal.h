@@ -34,6 +34,8 @@ struct AttnParams {
     int key_slab, value_slab;  // (depth - 1) * layers + layer
     float scale_log2;          // softmax scale * log2(e)
     int num_ctas;
+    bool short_ranges;         // attn_short_ranges
+    int block_weight;          // weight of a block tile in the split (set by attn_launch)
 };
 
 // Number of CTAs the attention kernel launches on `device` (a persistent
@@ -45,12 +47,22 @@ size_t attn_workspace_bytes(int device, int batch, int kv_heads, int rows_max, i
 void attn_workspace_layout(void *workspace, int batch, int kv_heads, int rows_max, int head_dim,
                            int num_ctas, AttnParams &p);
 
-// Launch the tcgen05 attention kernel and its split-K merge on `stream`, each
-// a programmatic dependent of the kernel before it; tm_q maps the queries
-// [B][max_block][Hq][D] with a {64, G, max_block, 1} box.
-// keys_e4m3 / values_e4m3: tm_k / tm_v map e4m3 prefix tiles (8-bit maps with
-// a {D, 1, 64, 1, 1} box, no swizzle) instead of bf16 ones.
-cudaError_t attn_launch(const AttnParams &p, int head_dim, bool keys_e4m3, bool values_e4m3,
+// Whether a call's ranges are short enough for the kernel of das_rows.cu.
+bool attn_short_ranges(int device, int batch, int kv_heads, int capacity, int head_dim,
+                       int rows_max, bool keys_e4m3, bool values_e4m3);
+
+// Launch an attention kernel (p.short_ranges: the one of das_rows.cu) and the
+// split-K merge on `stream`, each a programmatic dependent of the kernel before
+// it; tm_q maps the queries [B][max_block][Hq][D] with a {64, G, max_block, 1} box.
+// tm_k maps one 64-key prefix tile (bf16: one 64-column panel of it), tm_k2 two
+// consecutive ones (not with p.short_ranges), tm_v one (p.short_ranges and bf16:
+// one panel of it); keys_e4m3 / values_e4m3: 8-bit maps.
+cudaError_t attn_launch(AttnParams p, int head_dim, bool keys_e4m3, bool values_e4m3,
+                        const CUtensorMap &tm_k, const CUtensorMap &tm_k2, const CUtensorMap &tm_v,
+                        const CUtensorMap &tm_kb, const CUtensorMap &tm_vb,
+                        const CUtensorMap &tm_q, cudaStream_t stream);
+
+cudaError_t rows_launch(const AttnParams &p, int head_dim, bool keys_e4m3, bool values_e4m3,
                         const CUtensorMap &tm_k, const CUtensorMap &tm_v,
                         const CUtensorMap &tm_kb, const CUtensorMap &tm_vb,
                         const CUtensorMap &tm_q, cudaStream_t stream);
