@@ -113,6 +113,8 @@ size_t das_workspace_size(const das_kv_cache *cache, int num_q_heads, int max_bl
  *                  overlap in time
  * Device-side: prefix_len or block_len outside their ranges are clamped and
  * bit 1 of the workspace status word is set.
+ * A row with a score of NaN or +infinity (from its query or a key that it sees)
+ * gives NaN outputs and lse; other rows are unaffected.
  */
 das_status das_mature_v_attention(const das_kv_cache *cache, int layer, int key_depth,
                                   int value_depth, const int32_t *prefix_len,
@@ -278,7 +280,8 @@ size_t das_workspace_size_f8(const das_kv_cache_f8 *cache, int num_q_heads, int 
  * split into two or three 8-bit parts under a power of two per row (fp32
  * accumulation; two parts, at head_dim 128 with bf16 values, are exact for elements
  * down to about 2^-10 of the row's largest magnitude, three to 2^-17).
- * With e4m3 keys the queries must be finite; a row that is not gives NaN.
+ * With e4m3 keys the queries must be finite; a row that is not gives NaN (0 and lse
+ * -inf where its keys are widened and all its scores are -inf).
  */
 das_status das_mature_v_attention_f8(const das_kv_cache_f8 *cache, int layer, int key_depth,
                                      int value_depth, const int32_t *prefix_len,

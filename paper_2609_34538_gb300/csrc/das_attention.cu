@@ -1445,7 +1445,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                 // m + log2(l), l's exponent apart: m and it may cancel
                 const float e = (float)((int)(__float_as_uint(lsum) >> 23) - 127);
                 const float f = __uint_as_float((__float_as_uint(lsum) & 0x7fffffu) | 0x3f800000u);
-                const float lse = lsum > 3.4e38f ? INFINITY
+                const float lse = !(lsum <= 3.4e38f) ? lsum  // infinite or NaN
                                   : lsum > 0.f
                                       ? ((e - lds(nm_sm + 4 * r)) + __log2f(f)) * kLn2
                                       : -INFINITY;
@@ -1532,7 +1532,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
 // holding O_s / l_s and lse_s for the row:
 //   out = sum_s e^(lse_s - M) O_s / l_s / sum_s e^(lse_s - M),
 //   lse = M + ln sum_s e^(lse_s - M),  M = max_s lse_s,
-// and rows past the block get 0 and lse -inf.  The pair's segments are found
+// (NaN if any lse_s is) and rows past the block get 0 and lse -inf.  The pair's segments are found
 // from the lengths before griddepcontrol.wait (the attention grid this one
 // depends on started after every kernel that could write them had
 // completed); the partials are read after it, SEGS segments of each of the
@@ -1640,7 +1640,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32, merge_min_blocks<SEGS, RPW>(
         for (int r = 0; r < RPW; ++r) {
             float mn = M[r];
 #pragma unroll
-            for (int u = 0; u < SEGS; ++u) mn = fmaxf(mn, ls[r][u]);
+            for (int u = 0; u < SEGS; ++u) mn = max_nan(mn, ls[r][u]);
             if (mn == -INFINITY) continue;
             const float a = __expf(M[r] - mn);  // 0 while M is -inf
             L[r] *= a;
@@ -1667,7 +1667,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32, merge_min_blocks<SEGS, RPW>(
         else
             *reinterpret_cast<uint32_t *>(orow[r]) =
                 pack_bf16(acc[r][0] * inv, acc[r][VPL - 1] * inv);
-        if (lane == 0) *lrow[r] = L[r] > 0.f ? M[r] + __logf(L[r]) : -INFINITY;
+        if (lane == 0) *lrow[r] = L[r] == 0.f ? -INFINITY : M[r] + __logf(L[r]);
     }
 }
 

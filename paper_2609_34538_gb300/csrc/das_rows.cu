@@ -320,7 +320,9 @@ __device__ __forceinline__ void widen_tile(uint32_t src, uint32_t dst, int ct) {
 // falls below e4m3's smallest subnormal (2^-9), i.e. for elements below about
 // 2^-9 of the row's largest.  Thread ct of the 128 conversion threads takes
 // row ct / 2, dims [64 (ct % 2), +64); e is written to qexp[row].  A row of
-// zeros gives e = 0; the query must be finite.
+// zeros gives e = 0; a row with an infinity or NaN gives kNotFinite (its scores
+// are then NaN; the parts of an infinity would be finite).
+constexpr int kNotFinite = 1 << 20;
 __device__ __forceinline__ void split_q(uint32_t q, uint32_t hi, uint32_t lo, int *qexp, int ct) {
     const int row = ct >> 1, half = ct & 1;
     uint32_t w[32];
@@ -329,15 +331,14 @@ __device__ __forceinline__ void split_q(uint32_t q, uint32_t hi, uint32_t lo, in
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                      : "=r"(w[4 * c]), "=r"(w[4 * c + 1]), "=r"(w[4 * c + 2]), "=r"(w[4 * c + 3])
                      : "r"(q + half * (kRows * 128) + row * 128 + ((c ^ (row & 7)) << 4)));
-    float mx = 0.f;
+    uint32_t mb = 0;  // largest magnitude, as bits (a NaN's are the largest)
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-        mx = fmaxf(mx, fmaxf(fabsf(__uint_as_float(w[i] << 16)),
-                             fabsf(__uint_as_float(w[i] & 0xffff0000u))));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mb = max(mb, max((w[i] << 16) & 0x7fff0000u, w[i] & 0x7fff0000u));
+    mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, 1));
     int e = 0;
-    if (mx > 0.f && mx <= 3.4e38f) {
-        e = 7 - ((int)((__float_as_uint(mx) >> 23) & 0xffu) - 127);
+    if (mb != 0u && mb < 0x7f800000u) {
+        e = 7 - ((int)(mb >> 23) - 127);
         e = e < -120 ? -120 : (e > 120 ? 120 : e);
     }
     const float sc = __uint_as_float((uint32_t)(127 + e) << 23);
@@ -381,7 +382,7 @@ __device__ __forceinline__ void split_q(uint32_t q, uint32_t hi, uint32_t lo, in
                      "r"(l[4 * m + 1]), "r"(l[4 * m + 2]), "r"(l[4 * m + 3])
                      : "memory");
     }
-    if (half == 0) qexp[row] = e;
+    if (half == 0) qexp[row] = mb >= 0x7f800000u ? kNotFinite : e;
 }
 
 // Registers a thread of the query-split variant may use: 144 x 352 threads
@@ -961,7 +962,9 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                     const int qb = qs & 1;
                     wait(b_qsplit + 8 * qb, (uint32_t)((qs >> 1) & 1), abort_flag, p.status);
                     const int e = qexp[qb * kRows + row];
-                    row_scale = p.scale_log2 * __uint_as_float((uint32_t)(127 - e) << 23);
+                    row_scale = e == kNotFinite
+                                    ? __uint_as_float(0x7fc00000u)
+                                    : p.scale_log2 * __uint_as_float((uint32_t)(127 - e) << 23);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(b_qempty + 8 * qb);
                 }
@@ -1227,7 +1230,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                         }
                     }
                     const float inv = Lr > 0.f ? 1.f / Lr : 0.f;
-                    const float lse = L > 0.f ? (M + __log2f(L)) * kLn2 : -INFINITY;
+                    const float lse = L == 0.f ? -INFINITY : (M + __log2f(L)) * kLn2;
                     if (write) {
                         if (whole) {
                             uint16_t *orow = p.out + (((size_t)ws.b * p.max_block + irow) * p.Hq +
@@ -1307,7 +1310,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                         }
                     }
                     const float inv = Lr > 0.f ? 1.f / Lr : 0.f;
-                    const float lse = L > 0.f ? (M + __log2f(L)) * kLn2 : -INFINITY;
+                    const float lse = L == 0.f ? -INFINITY : (M + __log2f(L)) * kLn2;
                     if (write) {
                         if (whole) {
                             uint16_t *orow = p.out + (((size_t)ws.b * p.max_block + irow) * p.Hq +
@@ -1340,7 +1343,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                     asm volatile("bar.sync 1, 128;" ::: "memory");
                 } else {
                 const float inv = l_row_rnd > 0.f ? 1.f / l_row_rnd : 0.f;
-                const float lse = l_row > 0.f ? (m_ref + __log2f(l_row)) * kLn2 : -INFINITY;
+                const float lse = l_row == 0.f ? -INFINITY : (m_ref + __log2f(l_row)) * kLn2;
                 if (write) {
                     uint16_t *orow = p.out + (((size_t)ws.b * p.max_block + irow) * p.Hq +
                                               (size_t)ws.h * p.G + gq) * D + 32 * half;
