@@ -37,8 +37,8 @@
 //   conversion warps: the query split, and e4m3 V widened to f16 tiles.
 //   softmax warps: thread j takes key j's scores of its group's query rows from
 //     tensor memory, subtracts the rows' references (base 2; a reference only
-//     moves when a score exceeds it by 2^60, or 2^15 for f16 P: then O and the
-//     sums are rescaled in tensor memory), and writes P = 2^(s - m) as bf16 (f16
+//     moves when a score exceeds it by 2^8, or 2^12 for f16 P: then O and the sums
+//     are rescaled in tensor memory), and writes P = 2^(s - m) as bf16 (f16
 //     for widened values) into the swizzled, MN-major P buffer.  The sums of the
 //     fp32 weights (for the lse) stay per thread, in tensor memory, and are added
 //     up at a segment's end; the sum of the rounded weights normalises O, so that
@@ -69,19 +69,22 @@ namespace tc {
 namespace {
 
 constexpr int kPBufs = 2;            // P buffers
-// The reference of a row moves only when a score exceeds it by more than
-// 2^kRescale: P and its sums are floating point, so a low reference costs no
-// precision, and moving it costs a CTA about 4 us.  f16 P (widened values) must
-// stay below 2^16, bf16 P and the fp32 sums of P V far below 2^127.
-// A segment's first reference is the maximum over its first keys: where the scores
-// of a row are all alike, or few, its weights should lie at or just below 1 (bf16
-// holds 1 exactly, and its relative error is half as large just below 1 as just
-// above; with the first key's score alone the largest error of a test's output
-// rose from 9.5e-3 to 1.06e-2 of the row's rms).  32 keys for f16 P (fewer moves)
-// and for pairs of up to kRefTiles tiles, else 16 (us, 32 -> 16: the draft, verify,
-// accept and commit step of B2 92.2 -> 91.0, two calls of B4 P32768 173.1 -> 172.9).
-constexpr float kRescaleBf16 = 60.f, kRescaleF16 = 15.f;
-constexpr int kRefKeys = 32, kRefTiles = 9;
+// P = 2^(s - m + shift).  A row's reference m moves only when log2 P would pass kTop:
+// as in das_rows.cu by 2^8 for bf16 P, so that the fp32 sums of P V hold values up to
+// about 2^(127 - 8) over the number of keys, and a row's largest weights mostly sit at
+// or just below a reference (bf16 holds 1 exactly, and its relative error is half as
+// large just below 1 as just above).  Moving at 2^60 instead cost both: infinities
+// for values above about 2^60, and more error against 64 bits (batched 1.99e-3
+// against 1.95e-3, e4m3 keys B4 P16384 1.88e-3 against 1.84e-3).  f16 P (widened values)
+// holds 2^-25 to 2^16: kTop of 2^15, and a shift so that a long flat tail under one
+// strong key vanishes from O only below 2^-28 of it (e4m3 keys and values, two calls
+// of B8 ragged: shift 0 87.9 us, 3 89.6, 5 93.2, 7 98.5).
+// When a row moves, all rows of the group move up to their maximum over the step:
+// fewer moves, each of which costs a CTA about 1 us (ragged B8 D64 56.7 instead of
+// 61.4 us, e4m3 keys B4 P16384 86.0 instead of 89.5).
+// A segment's first reference is the maximum over its first kRefKeys keys.
+constexpr float kTopBf16 = 8.f, kTopF16 = 15.f, kShiftF16 = 3.f;
+constexpr int kRefKeys = 32;
 constexpr float kNoRef = 3e38f;      // -reference of a row without a finite score yet
 
 // Shared memory of one CTA.  A step is one or two consecutive 64-key tiles of
@@ -467,6 +470,17 @@ __device__ __forceinline__ void soft_sync(int group) {
         asm volatile("bar.sync 2, 128;" ::: "memory");
 }
 
+template <int NC>
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&x)[NC]) {
+#pragma unroll
+    for (int c = 0; c < NC; c += 16) {
+        float o[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) o[j] = x[c + j];
+        tmem_st16(taddr + c, o);
+    }
+}
+
 // The lane's columns from taddr: x, or what they hold plus x.  The stores are
 // waited for by the next call, or by whoever reads them.
 template <int NC>
@@ -478,13 +492,7 @@ __device__ __forceinline__ void tmem_accumulate(uint32_t taddr, float (&x)[NC], 
 #pragma unroll
         for (int j = 0; j < NC; j += 2) add2(x[j], x[j + 1], x[j], x[j + 1], o[j], o[j + 1]);
     }
-#pragma unroll
-    for (int c = 0; c < NC; c += 16) {
-        float o[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) o[j] = x[c + j];
-        tmem_st16(taddr + c, o);
-    }
+    tmem_st<NC>(taddr, x);
 }
 
 // NC values from shared memory into every lane's columns of tensor memory.
@@ -889,9 +897,6 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                 atomicOr(p.status, kStatusClamped);
     // an empty range (only when N < C) runs no loop below
 
-    // keys of a segment's first reference
-    auto ref_keys = [&](const Walk &w) { return VF8 || w.nt <= kRefTiles ? kRefKeys : kRefKeys / 2; };
-
     int drain_copy = -1;  // the last copy a conversion warp started, for the abort path's drain
     if (warp == kProducerWarp) {
         // ================================ producer ===============================
@@ -905,6 +910,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
         // =============================== S^T = K Q^T =============================
         const uint32_t id_s = idesc(128, N, 0, 0);
         const uint32_t id_s8 = idesc_e4m3(128, N);
+        const uint32_t id_r = idesc(64, kRefKeys, 0, 0), id_r8 = idesc_e4m3(64, kRefKeys);
         // descriptors are affine in the address: build each base once and add
         // (byte offset >> 4) for slots, panels and k-steps
         const uint64_t dk = sdesc(sbase, 16, 1024, kSw128);
@@ -935,7 +941,6 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
         for (int past = 0, seg = 0, k = 0, kf = 0; past < ntiles && ok; ++seg) {
             const Seg sc = segment<kConv>(w, ntiles - past);
             const int qb = seg & 1;
-            const uint32_t id_r = idesc(64, ref_keys(w), 0, 0), id_r8 = idesc_e4m3(64, ref_keys(w));
             ok = await(b_qfull, qb, seg >> 1);
             if (KF8) ok = ok && await(b_qsplit, qb, seg >> 1);
             for (int i = 0; i < sc.steps && ok; ++i, ++k) {
@@ -1146,6 +1151,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
         // hide each other's latencies; one group of 64 columns needed 255
         // registers and was slower on every 64-column case).
         constexpr int NC = Lt::kCols;
+        constexpr float kShift = VF8 ? kShiftF16 : 0.f, kTop = VF8 ? kTopF16 : kTopBf16;
         const int group = Lt::kGroups == 1 ? 0 : warp >> 2, key = threadIdx.x & 127;
         const int half = key >> 6, kidx = key & 63;  // tile of the step, key of the tile
         const int col0 = group * NC;
@@ -1225,7 +1231,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                     float x[kRefKeys];
                     tmem_ld<kRefKeys>(tmem + lane_base + (uint32_t)Lt::kRefCol, x);
                     const int r = (warp & 3) * 16 + lane - col0;  // lanes < 16
-                    const int nv = min(ref_keys(w), tile_keys(w, t0));
+                    const int nv = min(kRefKeys, tile_keys(w, t0));
                     const int lim = t0 == w.nt - 1 ? min(nv, (r + col0) / p.G + 1) : nv;
                     float m = -INFINITY;
 #pragma unroll
@@ -1234,7 +1240,9 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                         m *= f8s ? lds(sc_row + 4 * r) : p.scale_log2;
                         // a row with no finite score yet keeps a reference far below
                         // any; rows past the block weigh nothing and never move it
-                        sts(nm_sm + 4 * r, r >= rows_active ? -INFINITY : m == -INFINITY ? kNoRef : -m);
+                        sts(nm_sm + 4 * r, r >= rows_active  ? -INFINITY
+                                           : m == -INFINITY ? kNoRef
+                                                            : kShift - m);
                     }
                 }
                 soft_sync(group);
@@ -1250,9 +1258,9 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
             for (int c = 8; c < NC; c += 8)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) m4[j] = max3(m4[j], v[c + j], v[c + 4 + j]);
-            // a score far beyond its row's reference: the reference moves
+            // a score far beyond its row's reference: the references move
             const bool move =
-                soft_any(group, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) > (VF8 ? kRescaleF16 : kRescaleBf16));
+                soft_any(group, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) > kTop);
             const uint32_t pbuf = (uint32_t)((k & 1) * Lt::kPBytes);
             if (move) {  // the same in all of the group's warps
                 // the rows' maxima over the step, through the P buffer (free once
@@ -1275,8 +1283,8 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                                           fmaxf(lds(red + 8 * N), lds(red + 12 * N)));
                     const float old = lds(nm_sm + 4 * r);
                     float nm = old, alpha = 1.f;
-                    if (m + old > (VF8 ? kRescaleF16 : kRescaleBf16) && m != -INFINITY) {  // (old = -inf past the block)
-                        nm = -m;
+                    if (m + old > kShift && m != -INFINITY) {  // (old = -inf past the block)
+                        nm = kShift - m;
                         alpha = ex2(nm - old);
                     }
                     sts(nm_sm + 4 * r, nm);
@@ -1292,11 +1300,11 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                     tmem_wait_st();
 #pragma unroll 1
                     for (int c = 0; c < (D == 128 ? 3 : 2) * NC; c += 16) {
-                        float o[16];
                         const int at = c < NC       ? Lt::kSumCol
                                        : c < 2 * NC ? Lt::kOCol - NC
                                                     : Lt::kLCol - 2 * NC;
                         const uint32_t ta = tmem + lane_base + (uint32_t)(at + col0 + c);
+                        float o[16];
                         tmem_ld<16>(ta, o);
 #pragma unroll
                         for (int r = 0; r < 16; r += 4) {

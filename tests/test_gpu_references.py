@@ -1,0 +1,77 @@
+"""The rows' references (what is subtracted from the scores before the exponential):
+they move over a segment's steps, large values do not overflow the sums, and small
+weights under a strong early key are not lost."""
+import pytest
+import torch
+
+from tests.device_util import Call, assert_rows
+
+pytestmark = pytest.mark.gpu
+
+STORES = [(False, False), (True, False), (True, True), (False, True)]
+ROWS = [(1, 15), (4, 5), (4, 15)]  # (G, T): 16, 32 and 64 query columns
+
+
+def ramp(c, rise):
+    """Scores that rise by `rise` (natural units) over every 512 keys, and fall back:
+    whatever the split, a segment of more than 512 keys sees its rows' maxima grow at
+    several of its steps of 128."""
+    t = torch.arange(c.k.shape[1], device="cuda").remainder(512).float() / 32
+    c.k[..., 0] = t[None, :, None].to(c.k.dtype)  # 0 .. 16
+    c.q[..., 0] = rise / 16 * c.D ** 0.5
+    return c
+
+
+@pytest.mark.parametrize("kf8,vf8", STORES)
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("G,T", ROWS)
+def test_references_move_within_a_segment(kf8, vf8, D, G, T):
+    """24 pairs of 12000 keys: about 29 tiles a CTA, so that nearly every segment has a
+    dozen steps, and each rise of 60 (87 in base 2) moves the references at most of a
+    ramp's four steps: O, the sums and the rounded sums are rescaled after the first."""
+    c = ramp(Call([12000, 11937, 12001], [T, T, T - 1], G, 8, D, kf8, vf8, seed=1), 60.0)
+    out, lse = c.run()
+    assert_rows(out, lse, c.reference())
+    assert c.status() == 0
+
+
+@pytest.mark.parametrize("kf8,vf8", STORES)
+@pytest.mark.parametrize("D", [64, 128])
+def test_sharp_scores(kf8, vf8, D):
+    """Random scores of deviation 20 over segments of many steps."""
+    c = Call([12000, 11937, 12001], [13] * 3, 4, 8, D, kf8, vf8, seed=2, sharp=20.0)
+    out, lse = c.run()
+    assert_rows(out, lse, c.reference())
+
+
+@pytest.mark.parametrize("kf8", [False, True])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("G,T", ROWS)
+@pytest.mark.parametrize("P", [700, 12000])
+def test_large_values(kf8, D, G, T, P):
+    """bf16 values of about 2^100, under scores that exceed a segment's first by far:
+    the sums of P V stay finite (weights of up to 2^8, at most 2^15 keys near them)."""
+    c = ramp(Call([P] * 3, [T] * 3, G, 8, D, kf8, seed=4), 60.0)
+    c.v.mul_(2.0 ** 100)
+    c.vb.mul_(2.0 ** 100)
+    out, lse = c.run()
+    assert bool(out.isfinite().all())
+    assert_rows(out, lse, c.reference())
+
+
+@pytest.mark.parametrize("kf8,vf8", STORES)
+@pytest.mark.parametrize("D", [64, 128])
+def test_flat_tail_under_a_strong_key(kf8, vf8, D):
+    """One key of weight 1 and value 0, 16383 of weight 2^-25.5 and value 1 each: they are
+    the output.  160 pairs, so that a CTA has a whole pair's keys in one segment."""
+    c = Call([16384] * 40, [2] * 40, 4, 4, D, kf8, vf8, seed=5)
+    c.k.zero_()
+    c.kb.zero_()
+    c.q.zero_()
+    c.k[:, 0, :, 0] = 8.0
+    c.q[..., 0] = 25.5 * 0.6931 * D ** 0.5 / 8
+    c.v[:] = torch.ones((), device="cuda").to(c.v.dtype)
+    c.v[:, 0] = torch.zeros((), device="cuda").to(c.v.dtype)
+    c.vb.zero_()
+    out, lse = c.run()
+    assert_rows(out, lse, c.reference())
