@@ -37,7 +37,7 @@
 //   conversion warps: the query split, and e4m3 V widened to f16 tiles.
 //   softmax warps: thread j takes key j's scores of its group's query rows from
 //     tensor memory, subtracts the rows' references (base 2; a reference only
-//     moves when a score exceeds it by 2^8, or 2^15 for f16 P: then O and the sums
+//     moves when a score exceeds it by 2^8, or 2^12 for f16 P: then O and the sums
 //     are rescaled in tensor memory), and writes P = 2^(s - m) as bf16 (f16
 //     for widened values) into the swizzled, MN-major P buffer.  The sums of the
 //     fp32 weights (for the lse) stay per thread, in tensor memory, and are added
@@ -69,19 +69,21 @@ namespace tc {
 namespace {
 
 constexpr int kPBufs = 2;            // P buffers
-// P = 2^(s - m).  A row's reference m moves only when log2 P would pass kTop:
+// P = 2^(s - m + shift).  A row's reference m moves only when log2 P would pass kTop:
 // as in das_rows.cu by 2^8 for bf16 P, so that the fp32 sums of P V hold values up to
 // about 2^(127 - 8) over the number of keys, and a row's largest weights mostly sit at
 // or just below a reference (bf16 holds 1 exactly, and its relative error is half as
 // large just below 1 as just above).  Moving at 2^60 instead cost both: infinities
 // for values above about 2^60, and more error against 64 bits (batched 1.99e-3
-// against 1.95e-3, e4m3 keys B4 P16384 1.88e-3 against 1.84e-3).  f16 P (widened
-// values) must stay below 2^16.
+// against 1.95e-3, e4m3 keys B4 P16384 1.88e-3 against 1.84e-3).  f16 P (widened values)
+// holds 2^-25 to 2^16: kTop of 2^15, and a shift so that a long flat tail under one
+// strong key vanishes from O only below 2^-28 of it (e4m3 keys and values, two calls
+// of B8 ragged: shift 0 87.9 us, 3 89.6, 5 93.2, 7 98.5).
 // When a row moves, all rows of the group move up to their maximum over the step:
 // fewer moves, each of which costs a CTA about 1 us (ragged B8 D64 56.7 instead of
 // 61.4 us, e4m3 keys B4 P16384 86.0 instead of 89.5).
 // A segment's first reference is the maximum over its first kRefKeys keys.
-constexpr float kTopBf16 = 8.f, kTopF16 = 15.f;
+constexpr float kTopBf16 = 8.f, kTopF16 = 15.f, kShiftF16 = 3.f;
 constexpr int kRefKeys = 32;
 constexpr float kNoRef = 3e38f;      // -reference of a row without a finite score yet
 
@@ -1149,7 +1151,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
         // hide each other's latencies; one group of 64 columns needed 255
         // registers and was slower on every 64-column case).
         constexpr int NC = Lt::kCols;
-        constexpr float kTop = VF8 ? kTopF16 : kTopBf16;
+        constexpr float kShift = VF8 ? kShiftF16 : 0.f, kTop = VF8 ? kTopF16 : kTopBf16;
         const int group = Lt::kGroups == 1 ? 0 : warp >> 2, key = threadIdx.x & 127;
         const int half = key >> 6, kidx = key & 63;  // tile of the step, key of the tile
         const int col0 = group * NC;
@@ -1240,7 +1242,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                         // any; rows past the block weigh nothing and never move it
                         sts(nm_sm + 4 * r, r >= rows_active  ? -INFINITY
                                            : m == -INFINITY ? kNoRef
-                                                            : -m);
+                                                            : kShift - m);
                     }
                 }
                 soft_sync(group);
@@ -1281,8 +1283,8 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                                           fmaxf(lds(red + 8 * N), lds(red + 12 * N)));
                     const float old = lds(nm_sm + 4 * r);
                     float nm = old, alpha = 1.f;
-                    if (m + old > 0.f && m != -INFINITY) {  // (old = -inf past the block)
-                        nm = -m;
+                    if (m + old > kShift && m != -INFINITY) {  // (old = -inf past the block)
+                        nm = kShift - m;
                         alpha = ex2(nm - old);
                     }
                     sts(nm_sm + 4 * r, nm);

@@ -1,5 +1,6 @@
 """The rows' references (what is subtracted from the scores before the exponential):
-they move over a segment's steps, and large values do not overflow the sums."""
+they move over a segment's steps, large values do not overflow the sums, and small
+weights under a strong early key are not lost."""
 import pytest
 import torch
 
@@ -55,4 +56,22 @@ def test_large_values(kf8, D, G, T, P):
     c.vb.mul_(2.0 ** 100)
     out, lse = c.run()
     assert bool(out.isfinite().all())
+    assert_rows(out, lse, c.reference())
+
+
+@pytest.mark.parametrize("kf8,vf8", STORES)
+@pytest.mark.parametrize("D", [64, 128])
+def test_flat_tail_under_a_strong_key(kf8, vf8, D):
+    """One key of weight 1 and value 0, 16383 of weight 2^-25.5 and value 1 each: they are
+    the output.  160 pairs, so that a CTA has a whole pair's keys in one segment."""
+    c = Call([16384] * 40, [2] * 40, 4, 4, D, kf8, vf8, seed=5)
+    c.k.zero_()
+    c.kb.zero_()
+    c.q.zero_()
+    c.k[:, 0, :, 0] = 8.0
+    c.q[..., 0] = 25.5 * 0.6931 * D ** 0.5 / 8
+    c.v[:] = torch.ones((), device="cuda").to(c.v.dtype)
+    c.v[:, 0] = torch.zeros((), device="cuda").to(c.v.dtype)
+    c.vb.zero_()
+    out, lse = c.run()
     assert_rows(out, lse, c.reference())
