@@ -278,8 +278,9 @@ size_t das_workspace_size_f8(const das_kv_cache_f8 *cache, int num_q_heads, int 
  * e4m3 values enter the products exactly (widened).  e4m3 keys are widened
  * exactly too, or scored by 8-bit products of the stored keys with each query row
  * split into two or three 8-bit parts under a power of two per row (fp32
- * accumulation; two parts, at head_dim 128 with bf16 values, are exact for elements
- * down to about 2^-10 of the row's largest magnitude, three to 2^-17).
+ * accumulation).  Two parts, at head_dim 128 with bf16 values, are exact for elements
+ * down to 2^-9 of the row's largest magnitude and off by at most 2^-17 of it below;
+ * three, elsewhere, are exact down to 2^-23 and off by at most 2^-31 below.
  * With e4m3 keys the queries must be finite; a row that is not gives NaN (0 and lse
  * -inf where its keys are widened and all its scores are -inf).
  */

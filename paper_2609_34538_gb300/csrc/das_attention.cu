@@ -30,8 +30,8 @@
 // a producer, a P V and an S warp (+ four conversion warps for e4m3).
 //   S warp: loads K, a slot per step, and issues S^T (and, of a segment's first
 //     step, the scores of a few keys the other way round, from which each row's
-//     first reference is taken).  e4m3 keys: two e4m3 passes over the query
-//     rows split exactly into hi + lo, see split_q.
+//     first reference is taken).  e4m3 keys: two e4m3 or three e5m2 passes over
+//     the query rows split into that many parts, see split_q.
 //   producer warp: loads the query rows and V; the first steps' K too.
 //   P V warp: O^T += V^T P^T and the row sums, once P is in shared memory.
 //   conversion warps: the query split, and e4m3 V widened to f16 tiles.
@@ -120,8 +120,7 @@ struct Layout {
     static constexpr int kSBufs = KF8 && D == 128 && N == 64 ? 2 : 3;  // S buffers in tensor memory
     static constexpr int kQBytes = N * D * 2;    // one bf16 query buffer
     static constexpr int kQ8Bytes = N * D;       // one 8-bit query part
-    // (e4m3 keys) parts of the query split: the third where widening the keys,
-    // which is exact, was the alternative measured (split_q)
+    // (e4m3 keys) parts of the query split (split_q)
     static constexpr int kParts = VF8 || D == 64 ? 3 : 2;
     static constexpr int kPBytes = 2 * kTileKeys * N * 2;
     static constexpr int kVOff = kKSlots * kKBytes;
@@ -251,22 +250,21 @@ __device__ __forceinline__ void widen_tile(uint32_t src, uint32_t dst, int nvali
     }
 }
 
-// Exact split of the query rows for e4m3 keys.  Row r of the bf16 query
-// buffer q (128-byte-swizzled panels of [N rows][64 dims]) becomes two e4m3
-// rows hi, lo ([N rows][D] bytes, swizzled over the row) with
-//   2^e q = hi + lo,  e the largest with 2^e max_d |q_d| <= 448 (e4m3's
-// largest value; e clamped to +-120),
-// so that the row's largest element scales into (224, 448].  hi is 2^e q
-// rounded to e4m3 (4 significant bits) and lo the rounded remainder: a bf16
-// value has 8 significant bits, so the remainder fits e4m3 exactly unless it
-// falls below e4m3's smallest subnormal (2^-9), i.e. for elements below about
-// 2^-9 of the row's largest.  With PARTS = 3 what then remains (at most 2^-10) is
-// rounded to e5m2 (3 significant bits, to 2^-16) as a third part, which takes
-// the split's error below that of the fp32 sums (lse of e4m3 keys and values at
-// D = 64, against 64 bits: 8.3e-8 with two parts, 4.1e-8 with keys widened to
-// bf16).  128 / N threads share a row; qsc[row] becomes
-// the scale of the row's scores, scale_log2 2^-e (NaN for a row with an
-// infinity or NaN).
+// Split of the query rows for e4m3 keys.  Row r of the bf16 query buffer q
+// (128-byte-swizzled panels of [N rows][64 dims]) becomes PARTS 8-bit rows
+// ([N rows][D] bytes, swizzled over the row): 2^e q rounded, the remainder
+// rounded, and so on, with e the largest that keeps 2^e max_d |q_d| within the
+// type (e clamped to +-120).
+//   PARTS = 2: e4m3 (4 significant bits, largest 448, smallest 2^-9).  A bf16 value
+//     has 8 significant bits, so the parts are exact where the last of them is 2^-9
+//     or more: elements from 2^-9 of the row's largest on (which scales into
+//     (224, 448]).  Below, an element is off by at most 2^-10, 2^-17 of the largest.
+//   PARTS = 3: e5m2 (3 significant bits, largest 57344, smallest 2^-16): exact from
+//     2^-23 of the largest on, below off by at most 2^-31 of it.  Taken where the
+//     alternative was to widen the keys, which is exact.  (hi and lo as e4m3 and
+//     e5m2 for the third part alone was exact to 2^-14 only.)
+// 128 / N threads share a row; qsc[row] becomes the scale of the row's scores,
+// scale_log2 2^-e (NaN for a row with an infinity or NaN).
 template <int D, int N, int PARTS>
 __device__ __forceinline__ void split_q(uint32_t q, uint32_t parts, float *qsc, float scale_log2,
                                         int ct) {
@@ -289,7 +287,8 @@ __device__ __forceinline__ void split_q(uint32_t q, uint32_t parts, float *qsc, 
     for (int d = 1; d < kTpr; d <<= 1) mb = max(mb, __shfl_xor_sync(kFull, mb, d));
     int e = 0;
     if (mb != 0u) {
-        e = ((mb & 0x7fffffu) <= 0x600000u ? 8 : 7) - ((int)(mb >> 23) - 127);
+        constexpr int kTopExp = PARTS == 3 ? 15 : 8;  // the largest value is 1.75 2^kTopExp
+        e = ((mb & 0x7fffffu) <= 0x600000u ? kTopExp : kTopExp - 1) - ((int)(mb >> 23) - 127);
         e = e < -120 ? -120 : (e > 120 ? 120 : e);
     }
     const float sc = __uint_as_float((uint32_t)(127 + e) << 23);
@@ -303,7 +302,7 @@ __device__ __forceinline__ void split_q(uint32_t q, uint32_t parts, float *qsc, 
 #pragma unroll
             for (int z = 0; z < PARTS; ++z) {  // the next part of what is left
                 uint32_t c2, f2;
-                if (z < 2)
+                if (PARTS == 2)
                     asm("{\n .reg .b16 t;\n cvt.rn.satfinite.e4m3x2.f32 t, %2, %3;\n"
                         " cvt.u32.u16 %0, t;\n cvt.rn.f16x2.e4m3x2 %1, t;\n}"
                         : "=r"(c2), "=r"(f2)
@@ -909,8 +908,9 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
     } else if (warp == kSWarp) {
         // =============================== S^T = K Q^T =============================
         const uint32_t id_s = idesc(128, N, 0, 0);
-        const uint32_t id_s8 = idesc_e4m3(128, N);
-        const uint32_t id_r = idesc(64, kRefKeys, 0, 0), id_r8 = idesc_e4m3(64, kRefKeys);
+        constexpr uint32_t kE5 = Lt::kParts == 3 ? 1u : 0u;  // the query parts are e5m2
+        const uint32_t id_s8 = idesc_e4m3(128, N) | kE5 << 10;
+        const uint32_t id_r = idesc(64, kRefKeys, 0, 0), id_r8 = idesc_e4m3(64, kRefKeys) | kE5 << 7;
         // descriptors are affine in the address: build each base once and add
         // (byte offset >> 4) for slots, panels and k-steps
         const uint64_t dk = sdesc(sbase, 16, 1024, kSw128);
@@ -957,9 +957,8 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                 if (elect_one()) {
                     const uint32_t dS = tmem + (uint32_t)(rs.slot * N), dR = tmem + Lt::kRefCol;
                     const uint32_t slot = (uint32_t)(ru.slot * Lt::kKBytes) >> 4;
-                    // hi K^T, then lo K^T (, then lo2 K^T), 32 elements (32 bytes) per
-                    // MMA (the third part is e5m2: B of S^T, A of the reference scores);
-                    // bf16: panel kk / 4, then 16 elements within the 128-byte row
+                    // the parts' K^T one after the other, 32 elements (32 bytes) per MMA
+                    // (the queries are B of S^T, A of the reference scores); bf16: panel kk / 4, then 16 elements within the 128-byte row
                     const bool f8 = KF8 && 2 * i < sc.pairs;
                     auto key8 = [&](int kk) { return dk8 + (uint64_t)(slot + kk % (D / 32) * 2); };
                     auto qry8 = [&](int kk) {
@@ -977,8 +976,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                         if (f8) {
 #pragma unroll
                             for (int kk = 0; kk < Lt::kParts * (D / 32); ++kk)
-                                mma_f8(dR, qry8(kk), key8(kk),
-                                       kk / (D / 32) < 2 ? id_r8 : id_r8 | 1u << 7, kk > 0);
+                                mma_f8(dR, qry8(kk), key8(kk), id_r8, kk > 0);
                         } else {
 #pragma unroll
                             for (int kk = 0; kk < D / 16; ++kk)
@@ -989,8 +987,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                     if (f8) {
 #pragma unroll
                         for (int kk = 0; kk < Lt::kParts * (D / 32); ++kk)
-                            mma_f8(dS, key8(kk), qry8(kk),
-                                   kk / (D / 32) < 2 ? id_s8 : id_s8 | 1u << 10, kk > 0);
+                            mma_f8(dS, key8(kk), qry8(kk), id_s8, kk > 0);
                     } else {
 #pragma unroll
                         for (int kk = 0; kk < D / 16; ++kk)

@@ -12,11 +12,11 @@ from tests.gpu_util import LSE_ABS
 # U sum w_j |v_j - o|, which the weighted deviation of the values bounds.  A score off
 # by d moves a weight by the factor e^d: d is below the lse's bound.
 U = 2.0 ** -8
-SUMS = 2.0 ** -21  # error of an fp32 sum of up to 128 products, of the factors' norms
+SUMS = 2.0 ** -21  # error of an fp32 sum of up to 128 products, of their magnitudes' sum
 # The largest error of an element of a split query, of its row's largest element:
-# two parts end at e4m3's smallest subnormal 2^-9 (error 2^-10) with the largest
-# above 2^7; three end at e5m2's 2^-16, whose 3 bits leave 2^-14 of what is below 2^-10.
-SPLIT = {2: 2.0 ** -17, 3: 2.0 ** -21}
+# two parts end at e4m3's smallest value 2^-9 (error 2^-10) with the largest element
+# at 2^7 or above; three end at e5m2's 2^-16 with the largest above 2^14.
+SPLIT = {2: 2.0 ** -17, 3: 2.0 ** -31}
 
 
 class Call:
@@ -96,17 +96,17 @@ class Call:
             out[b, :t], dev[b, :t] = rows(o), rows(w @ V.square() - o.square())
             lse[b, :, :t] = l.reshape(H * G, t)
         # a score's error (natural units): fp32 sums of the products, and the part of a
-        # split query that is dropped, per key times the norms that bound the sums
+        # split query that is dropped times the keys
         off = torch.zeros(lse.shape, dtype=torch.float64, device="cuda")
         for b, (p, t) in enumerate(zip(self.P, self.T)):
             if t:
                 K = torch.cat([self.k[b, :p].double(), self.kb[b, :t].double()])
-                n2, n1 = K.norm(dim=-1).amax(0), K.abs().sum(-1).amax(0)  # [H]
-                q = self.q[b, :t].double().reshape(t, H, G, D)
-                d = SUMS * q.norm(dim=-1) * n2[:, None]
+                K = K.abs().permute(1, 2, 0)  # [H][D][keys]
+                q = self.q[b, :t].double().abs().reshape(t, H, G, D).permute(1, 2, 0, 3)
+                d = SUMS * (q.reshape(H, G * t, D) @ K).amax(-1)
                 if self.kf8:
-                    d = d + self.split * q.abs().amax(-1) * n1[:, None]
-                off[b, :, :t] = d.reshape(t, H * G).T
+                    d = d + self.split * q.reshape(H, G * t, D).amax(-1) * K.sum(1).amax(-1)[:, None]
+                off[b, :, :t] = d.reshape(H * G, t)
         off = LSE_ABS + off * (scale if scale > 0 else 1 / math.sqrt(D))
         w = 2 * off.permute(0, 2, 1)[..., None]
         return out, lse, 1.01 * ((U + w) * dev.clamp(min=0).sqrt() + U * out.abs()), off
