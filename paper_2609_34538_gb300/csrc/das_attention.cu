@@ -208,48 +208,6 @@ struct Ring {
     }
 };
 
-// Widen an e4m3 value tile [64 keys][D] (row-major, as the 8-bit TMA box
-// lands) into the f16 tile the P V MMAs read: D / 64 panels of [64 keys][128
-// bytes], 16-byte chunk j of key r at (j ^ (r % 8)) * 16 (128-byte swizzle).
-// Every e4m3 value is exactly an f16 value, so one conversion per pair does
-// it (bf16 took four).  Keys from nvalid on (anything, NaN included) become
-// zeros.  The 128 conversion threads (ct = 0..127) each take 16-element chunks.
-template <int D>
-__device__ __forceinline__ void widen_tile(uint32_t src, uint32_t dst, int nvalid, int ct) {
-    constexpr int kChunks = kTileKeys * D / 16;
-#pragma unroll
-    for (int i = 0; i < kChunks / (kConvWarps * 32); ++i) {
-        const int c = ct + i * kConvWarps * 32;
-        // Chunk c: 16 elements jj of a 64-column panel of a key.  The 8 lanes
-        // of a quarter warp (one shared-memory wavefront of 16-byte accesses)
-        // take two keys of opposite parity, so their loads (rows of D bytes)
-        // and their swizzled stores each touch 8 distinct 16-byte bank groups.
-        const int jj = c & 3;
-        const int pnl = D == 128 ? (c >> 2) & 1 : 0;
-        const int key = D == 128 ? ((c >> 4) << 1) + (pnl ^ ((c >> 3) & 1)) : c >> 2;
-        uint32_t w[4];
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
-                     : "r"(src + key * D + pnl * 64 + jj * 16));
-        const uint32_t row = dst + pnl * 8192 + key * 128;
-        const bool keep = key < nvalid;
-        uint32_t h[8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n cvt.rn.f16x2.e4m3x2 %0, l;\n"
-                " cvt.rn.f16x2.e4m3x2 %1, h;\n}\n"
-                : "=r"(h[2 * u]), "=r"(h[2 * u + 1])
-                : "r"(keep ? w[u] : 0u));
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                             row + (((2 * jj + u) ^ (key & 7)) << 4)),
-                         "r"(h[4 * u]), "r"(h[4 * u + 1]), "r"(h[4 * u + 2]), "r"(h[4 * u + 3])
-                         : "memory");
-    }
-}
-
 // Split of the query rows for e4m3 keys.  Row r of the bf16 query buffer q
 // (128-byte-swizzled panels of [N rows][64 dims]) becomes PARTS 8-bit rows
 // ([N rows][D] bytes, swizzled over the row): 2^e q rounded, the remainder
@@ -1128,7 +1086,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, N>::kThreads, 1)
                 } else {
                     const int vs = vt % VS;
                     if (!await(b_vfull, vs, vt / VS)) break;
-                    widen_tile<D>(sbase + Lt::kVOff + vs * Lt::kVBytes, dst, tile_keys(w, w.t), ct);
+                    widen_f16<D>(sbase + Lt::kVOff + vs * Lt::kVBytes, dst, tile_keys(w, w.t), ct);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) {

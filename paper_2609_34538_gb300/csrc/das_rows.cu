@@ -11,7 +11,9 @@
 //                (e4m3 keys at D = 128: two e4m3 passes over the query rows
 //                split exactly into hi + lo, see split_q)
 //   O += P V     tcgen05.mma M=64 N=D K=64   -> O in TMEM
-//   l += P 1     tcgen05.mma M=64 N=8 K=64   -> the rounded row sums
+//   2 l += P 2   tcgen05.mma M=64 N=8 K=64   -> the rounded row sums, doubled
+// e4m3 values are widened to f16 and meet f16 weights (a rounding of 2^-11 where bf16
+// has 2^-8); all other operands are bf16 (e4m3 keys where they are not split: widened).
 // An M=64 MMA puts row r in TMEM lane 32 (r / 16) + r % 16: softmax warp w owns
 // rows 16w..16w+15 and two threads share a row.  A row's reference max moves only
 // when a score exceeds it by more than 2^8.  Pairs of at most 16 (32) query rows
@@ -34,8 +36,9 @@ constexpr int kConvWarp0 = kSoftWarps + 3;    // e4m3 -> bf16 widening, query sp
 constexpr int kRows = 64;            // M of every MMA (query rows per pair)
 constexpr int kSBufs = 4;            // S buffers in tensor memory
 constexpr int kTmemCols = 512;       // S buffers [0, 64 kSBufs), O [64 kSBufs, 64 kSBufs + D),
-                                     // then 8 columns whose first is the rounded row sum
+                                     // then 8 columns whose first is twice the rounded row sum
 constexpr float kRescaleLog2 = 8.f;  // move the reference max only beyond 2^8
+constexpr float kShiftF16 = 7.f;     // f16 weights are 2^7 larger: f16 holds 2^-25 to 2^16
 
 // 32 columns of S for the calling thread (16 lanes x 2 halves): thread t < 16
 // of a warp gets TMEM lane t, columns [c, c + 32), thread t + 16 the same lane,
@@ -175,7 +178,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) 
 //     e per row (see split_q), and S = (hi + lo) K^T is two e4m3 products
 //     accumulated in fp32, 2^e times the bf16 product.  The pair's block
 //     tile (bf16 keys) has a bf16 key buffer of its own and bf16 MMAs.
-//   otherwise: the conversion warps widen every e4m3 tile into bf16 tiles, in
+//   otherwise: the conversion warps widen every e4m3 tile (keys to bf16, values to f16), in
 //     the 128-byte-swizzled layout the MMAs read, held in a ring of kConvSlots
 //     slots (tile j in slot j % kConvSlots) rather than one per stage: the
 //     smaller stages then fit 6 (or 7) deep instead of 4, which is what keeps
@@ -214,9 +217,10 @@ struct Layout {
         kQSplit ? kTileBytes + 4 * kQ8Bytes : kConvSlots * kConvBytes;
     static constexpr int kQOff = kConvOff + kExtraBytes;
     static constexpr int kPOff = kQOff + 2 * kQBytes;
-    // the B operand of the row-sum MMA: [8][64] bf16, row 0 ones, 128-byte swizzled
-    static constexpr int kOnesOff = kPOff + 2 * kPBytes;
-    static constexpr int kBarOff = kOnesOff + 1024;
+    // the B operand of the row-sum MMA: [8][64], row 0 twos (0x4000 is 2 as bf16 and as
+    // f16: the sums come doubled, which is exact), 128-byte swizzled
+    static constexpr int kTwosOff = kPOff + 2 * kPBytes;
+    static constexpr int kBarOff = kTwosOff + 1024;
     // barriers: full[kStages], empty[kStages], qfull[2], qempty[2],
     // sready[kSBufs], sfree[kSBufs], pready[2], pvdone[2], drain[2],
     // cready[kConvSlots], kfree[kConvSlots], vfree[kConvSlots], qsplit[2], bkfree
@@ -270,7 +274,7 @@ __device__ __forceinline__ uint32_t e4m3x2_to_bf16x2(uint32_t a) {
     return r;
 }
 
-// Widen an e4m3 tile [64 keys][D] (row-major, as the 8-bit TMA box lands)
+// Widen an e4m3 key tile [64 keys][D] (row-major, as the 8-bit TMA box lands)
 // into the bf16 tile the MMAs read: D / 64 panels of [64 keys][128 bytes],
 // 16-byte chunk j of key r at (j ^ (r % 8)) * 16 (128-byte swizzle).  The 128
 // conversion threads (ct = 0..127) each take 16-element chunks.
@@ -506,11 +510,11 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
         len_sm[lane0] = lane0 < p.B ? len_cg(p.prefix_len, lane0, p.capacity) : 0;
         len_sm[32 + lane0] = lane0 < p.B ? len_cg(p.block_len, lane0, p.max_block) : 0;
     }
-    if (threadIdx.x < 64) {  // the row-sum MMA's B operand: row 0 of [8][64] bf16 ones
-        const uint32_t one2 = threadIdx.x < 8 ? 0x3F803F80u : 0u;
+    if (threadIdx.x < 64) {  // the row-sum MMA's B operand: row 0 of [8][64] twos
+        const uint32_t two2 = threadIdx.x < 8 ? 0x40004000u : 0u;
         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
-                         sbase + Lt::kOnesOff + threadIdx.x * 16),
-                     "r"(one2)
+                         sbase + Lt::kTwosOff + threadIdx.x * 16),
+                     "r"(two2)
                      : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -726,9 +730,10 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
         const uint64_t dkb = sdesc(sbase + Lt::kBlkKOff, 16, 1024, kSw128);
         const uint64_t dv0 = sdesc(v_src(0, 0), 8192, 1024, kSw128);
         const uint64_t dp0 = sdesc(sbase + Lt::kPOff, 16, 1024, kSw128);
-        // rounded row sums: D[64][8] += P[64][64] ones[8][64]^T, column 0 = sum of P
-        const uint64_t d1 = sdesc(sbase + Lt::kOnesOff, 16, 1024, kSw128);
+        // rounded row sums: D[64][8] += P[64][64] twos[8][64]^T, column 0 = twice the sum of P
+        const uint64_t d1 = sdesc(sbase + Lt::kTwosOff, 16, 1024, kSw128);
         const uint32_t id_l = idesc(kRows, 8, 0, 0);
+        const uint32_t id_pv16 = idesc_f16(kRows, D, 0, 1), id_l16 = idesc_f16(kRows, 8, 0, 0);
         bool ok = true;
         if (warp == kSWarp) {
             Walk wsn = w0;
@@ -811,15 +816,16 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                     const uint64_t a0 = dp0 + (uint64_t)(((k & 1) * Lt::kPBytes) >> 4);
                     const uint64_t b0 = dv0 + (uint64_t)((v_src(s, k) - v_src(0, 0)) >> 4);
                     const uint32_t dO = tmem + kSBufs * kTileKeys;
+                    const bool f16 = VF8 && wm.t < wm.nt - 1;  // widened values
 #pragma unroll
                     for (int kk = 0; kk < kTileKeys / 16; ++kk)
                         mma(dO, a0 + (uint64_t)((kk * 32) >> 4),
-                            b0 + (uint64_t)((kk * 2048) >> 4), id_pv,
+                            b0 + (uint64_t)((kk * 2048) >> 4), f16 ? id_pv16 : id_pv,
                             (!first || kk > 0) ? 1u : 0u);
 #pragma unroll
                     for (int kk = 0; kk < kTileKeys / 16; ++kk)
                         mma(dO + D, a0 + (uint64_t)((kk * 32) >> 4), d1 + (uint64_t)((kk * 32) >> 4),
-                            id_l, (!first || kk > 0) ? 1u : 0u);
+                            f16 ? id_l16 : id_l, (!first || kk > 0) ? 1u : 0u);
                     mma_commit(b_pvdone + 8 * (int)(k & 1));
                     mma_commit(b_empty + 8 * s);
                     if (VF8) mma_commit(b_vfree + 8 * (int)(k % kSlots));
@@ -862,7 +868,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
             walk_next(p, wc);
         }
     } else if (Lt::kConv && warp >= kConvWarp0) {
-        // ============================ e4m3 -> bf16 ===============================
+        // ======================== e4m3 -> bf16 keys, f16 values ==================
         // Widen every prefix tile's e4m3 K (and V) into its ring slot once it
         // has landed and the slot is free, then hand the tile to the S warp
         // (cready).  A block tile's K (V) is bf16 already: for a ring operand
@@ -910,7 +916,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
             if (VF8) {
                 ok = slot_free(b_vfree, j);
                 if (!ok) break;
-                widen_tile<D>(sbase + s * Lt::kStageBytes + Lt::kKBytes, v_src(s, j), ct);
+                widen_f16<D>(sbase + s * Lt::kStageBytes + Lt::kKBytes, v_src(s, j), kTileKeys, ct);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -1026,7 +1032,8 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                                       fmaxf(m11[9], m11[10]));
                 mt = full_tile ? m * scale : m;
             }
-            mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 16));
+            // (f16 weights) 2^kShiftF16 times what they would be: the reference is that much lower
+            mt = fmaxf(mt, __shfl_xor_sync(kFull, mt, 16)) - (VF8 ? kShiftF16 : 0.f);
             if (first) {
                 m_ref = mt;
             } else {
@@ -1070,7 +1077,9 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
             for (int j = 0; j < kVals; ++j) v[j] = ex2(v[j]);
             uint32_t w[kVals / 2];
 #pragma unroll
-            for (int e = 0; e < kVals / 2; ++e) w[e] = pack_bf16(v[2 * e], v[2 * e + 1]);
+            for (int e = 0; e < kVals / 2; ++e)
+                w[e] = VF8 && !block_tile ? pack_f16(v[2 * e], v[2 * e + 1])
+                                          : pack_bf16(v[2 * e], v[2 * e + 1]);
             // P buffer (k & 1) is free once P V of tile k-2, its last reader, is done
             // (pvdone[k & 1] completes once per P V of tiles with that parity)
             if (k >= 2) wait(b_pvdone + 8 * (int)(k & 1), (uint32_t)(((k - 2) >> 1) & 1), abort_flag,
@@ -1151,7 +1160,7 @@ __global__ void __launch_bounds__(Layout<D, KF8, VF8, NC>::kThreads, 1)
                         : "=r"(r)
                         : "r"(tmem + lane_base + (uint32_t)(kSBufs * kTileKeys + D))
                         : "memory");
-                    l_rnd = __uint_as_float(r);
+                    l_rnd = 0.5f * __uint_as_float(r);
                 }
                 const float l_row_rnd = l_rnd + __shfl_xor_sync(kFull, l_rnd, 16);
                 const int gq = qrow % p.G;
