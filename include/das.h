@@ -113,6 +113,11 @@ size_t das_workspace_size(const das_kv_cache *cache, int num_q_heads, int max_bl
  *                  overlap in time
  * Device-side: prefix_len or block_len outside their ranges are clamped and
  * bit 1 of the workspace status word is set.
+ * Values (of the cache and the block) of magnitude above about 2^(119 - log2(keys))
+ * may overflow the fp32 sums.  Which of two kernels serves a call depends on batch,
+ * heads, head_dim, max_block, element types and the cache's capacity; the results of
+ * both have the same accuracy, but not the same last bits.  (bf16 keys and values at
+ * head_dim 128: one kernel, the same bits under any capacity.)
  * A row with a score of NaN or +infinity (from its query or a key that it sees)
  * gives NaN outputs and lse; other rows are unaffected.
  */
@@ -275,12 +280,14 @@ size_t das_workspace_size_f8(const das_kv_cache_f8 *cache, int num_q_heads, int 
  * (depths below R, e4m3), so Eqs. 2-3 are evaluated on the stored values.
  * key_depth = value_depth = d is the verify attention of depth d (Sec. 3.4).
  * All other arguments, results and limits as das_mature_v_attention.
- * e4m3 values enter the products exactly (widened).  e4m3 keys are widened
- * exactly too, or scored by 8-bit products of the stored keys with each query row
- * split into two or three 8-bit parts under a power of two per row (fp32
- * accumulation).  Two parts, at head_dim 128 with bf16 values, are exact for elements
- * down to 2^-9 of the row's largest magnitude and off by at most 2^-17 of it below;
- * three, elsewhere, are exact down to 2^-23 and off by at most 2^-31 below.
+ * e4m3 values enter the products exactly (widened to f16, with f16 weights).  e4m3
+ * keys are scored by 8-bit products with each query row split into two or three 8-bit
+ * parts under a power of two per row (fp32 accumulation), or widened, which is exact:
+ *   head_dim 128 with bf16 values: two parts, exact for elements down to 2^-9 of the
+ *     row's largest magnitude and off by at most 2^-17 of it below;
+ *   otherwise: widened while batch and capacity keep the ranges short (the choice of
+ *     kernel, see das_mature_v_attention), else three parts, exact down to 2^-23 and
+ *     off by at most 2^-31 below.
  * With e4m3 keys the queries must be finite; a row that is not gives NaN (0 and lse
  * -inf where its keys are widened and all its scores are -inf).
  */

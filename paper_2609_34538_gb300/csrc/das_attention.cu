@@ -44,12 +44,13 @@
 //     up at a segment's end; the sum of the rounded weights normalises O, so that
 //     the output is a convex combination of the values with exactly the
 //     weights the tensor core used.
-// Measured (us per call, the kernel with query rows in the lanes -> this one,
-// each with its merge): decode B1 H32/32 P4096 T8 16.7 -> 16.1, B16 ragged P
-// 1024-8192 60.2 -> 58.6, B4 P32768 T16 86.4 -> 86.9, ragged D = 64 B8 32.1 -> 26.4,
-// e4m3 keys B4 P16384 46.2 -> 42.0, e4m3 keys and values B8 ragged 58.1 -> 41.0.
-// Bound by DRAM on the long bf16 calls (6.2 TB/s with all fixed costs), by the
-// softmax step (about 2000 cycles) where keys and values are e4m3.
+// It serves 64-wide heads and e4m3 operands over long ranges; bf16 calls with 128-wide
+// heads, and short ranges, take the kernel of das_rows.cu (attn_short_ranges).
+// Measured (us per call with its merge, das_rows.cu's kernel -> this one): ragged B8
+// D64 29.6 -> 27.9, e4m3 keys B4 P16384 43.6 -> 42.3, e4m3 keys and values B8 ragged
+// 51.1 -> 40.6.  Bound by the softmax step (about 2000 cycles) where keys and values
+// are e4m3, and everywhere by how well the roles' code fits the instruction caches:
+// warps stand for want of an instruction as long as they wait for anything else.
 //
 // The kernel is launched as a programmatic dependent of the previous kernel
 // in the stream: barrier set-up, the tensor-memory allocation, the work plan
@@ -98,10 +99,9 @@ constexpr float kNoRef = 3e38f;      // -reference of a row without a finite sco
 //   bf16 tiles are D / 64 panels of 128-byte rows, 128-byte swizzled; e4m3 key
 //   tiles are rows of D bytes, swizzled over the row (128 or 64 bytes), e4m3
 //   value tiles plain rows.
-// Ring depths, measured (us per two calls): V 4 tiles against 5 at D = 128 bf16,
-// B4 P32768 169.9 / 170.5, decode 32.0 / 32.6 (more loads in flight than needed
-// delay the ones needed first); K 3 slots against 2 for N = 16, decode 32.1 /
-// 32.5; S buffers: as many as tensor memory holds, a K slot is free once S is.
+// Ring depths: V 4 tiles at D = 128 (5 were 0.4 % slower: more loads in flight than
+// needed delay the ones needed first); K 3 slots or, for wide bf16 steps, as many as
+// fit; S buffers: as many as tensor memory holds, a K slot is free once S is.
 template <int D, bool KF8, bool VF8, int N>
 struct Layout {
     static_assert(N == 16 || N == 32 || N == 64, "query columns: 16, 32 or 64");
@@ -126,7 +126,7 @@ struct Layout {
     static constexpr int kVOff = kKSlots * kKBytes;
     static constexpr int kWOff = kVOff + kVSlots * kVBytes;
     static constexpr int kQOff = kWOff + kWSlots * kTileBytes;
-    static constexpr int kQ8Off = kQOff + 2 * kQBytes;  // hi, lo (, lo2)
+    static constexpr int kQ8Off = kQOff + 2 * kQBytes;  // the parts
     static constexpr int kPOff = kQ8Off + (KF8 ? kParts * kQ8Bytes : 0);
     // (D = 64) 16 keys x 64 ones (bf16, then f16): the second half of the P V A operand
     static constexpr int kOnesOff = kPOff + kPBufs * kPBytes;
@@ -530,11 +530,9 @@ __device__ __forceinline__ float inverse(float x) {
 
 // Registers a thread may use, so that a merge CTA (one warp in each of the SM's
 // four register files of 512 x 32) fits beside the attention CTA: 192 with 7
-// warps (two a file) leave 128, 128 with 11 (three a file) too.  bf16 with N = 64
-// would spill at 128 (B16 ragged 241.0 instead of 238.2 us): 144 leave 80, enough
-// for all merge variants but the largest.  15 warps (four a file) leave no
-// room at 128, and fewer would spill.  Where the merge CTA did not fit, a
-// draft, verify, accept and commit step of B2 took 98.7 us instead of 93.8.
+// warps (two a file) leave 128, 128 with 11 (three a file) too.  bf16 with N = 64 takes
+// 144 (44 bytes spilled; at 128 more), which leave 80, enough for all merge variants but
+// the largest.  15 warps (four a file) leave no room at 128, and fewer would spill.
 template <int D, bool KF8, bool VF8, int N>
 constexpr int kRegCap = Layout<D, KF8, VF8, N>::kThreads <= 224 ? 192
                         : Layout<D, KF8, VF8, N>::kConv || N < 64 ? 128
@@ -1770,7 +1768,7 @@ cudaError_t launch_attn(const AttnParams &p, int head_dim, bool keys_e4m3, bool 
     if (head_dim == 128) {
         if (keys_e4m3)
             return values_e4m3 ? DAS_LAUNCH(128, true, true) : DAS_LAUNCH(128, true, false);
-        return values_e4m3 ? DAS_LAUNCH(128, false, true) : DAS_LAUNCH(128, false, false);
+        if (values_e4m3) return DAS_LAUNCH(128, false, true);
     }
     if (head_dim == 64) {
         if (keys_e4m3) return values_e4m3 ? DAS_LAUNCH(64, true, true) : DAS_LAUNCH(64, true, false);
@@ -1795,32 +1793,48 @@ int attn_grid_size(int device) {
     return sms;
 }
 
-// Whether a call takes the kernel for short ranges (das_rows.cu).  The transposed
-// kernel costs less per tile and 0.3 to 1.5 us more per segment, so it is taken
-// where the average segment, tiles / (pairs + CTAs), is long enough.  The prefix
-// lengths are the device's; the capacity bounds them.  Measured, time of the
-// short-range kernel over the transposed one's at that many tiles a segment:
-//   bf16 D = 128, N = 16: 1.6 0.95, 3.8 1.03, 5.7 1.01, 12 1.06;  N = 32 and 64: 3.2 0.96,
-//     5.7 0.96, 9.8 1.00, 10 1.03
-//   bf16 D = 64, N = 16: 1.6 1.01, 5.7 1.09, 12 1.38;  wider: 3.2 0.88, 5.7 0.95, 9.8 1.00
-//   e4m3 keys D = 128, N = 16: 1.6 1.09, 5.7 1.05, 18 1.14;  wider: 3.2 0.93, 5.7 0.99, 9.8 1.02
-//   e4m3 keys and values D = 128, N = 16: 1.6 1.01, 5.7 1.20, but over 256 pairs 3.8 0.91,
-//     6 0.92, over 512 12 1.20;  wider: 5.1 0.92, 9.8 1.04, 10 0.91 (256 pairs)
-//   the same at D = 64, N = 16: 5.7 0.95, 12 1.11, 18 1.31;  wider: 9.8 0.93, 10 0.88
+// Whether a call takes the kernel of das_rows.cu.  The transposed kernel costs less per
+// tile and up to 3 us more per call (a segment's first scores wait for a whole step,
+// its first references and its end take barriers), so it wins where the average
+// segment, tiles / (pairs + CTAs), is long.  The prefix lengths are the device's, and
+// a server's cache is longer than most of its prefixes; the capacity bounds them.  So
+// the lines lie at twice the segments where the two kernels break even: no call over
+// a cache at least half full is slower.  Below, at the least segments, the transposed
+// kernel takes up to 1.15 (16 columns) and 1.4 (64) times as long.  (Both in one kernel,
+// chosen by the lengths, cost each of them up to 10 to 25 %: their code is more than
+// the instruction caches hold well.)  Measured, time of das_rows.cu's kernel over the
+// transposed one's at that many tiles a segment (few: at most a pair a CTA / many):
+//   bf16 keys and values, D = 64: 16 columns 2.0 0.94, 5.0 1.08, 11 1.11, 33 1.28; 32: 5.0 0.96,
+//     11 1.02, 33 1.21; 64: 7.1 0.93, 19 1.01, 33 1.09
+//   the same at D = 128: 16: 0.6 0.90, 5.0 1.05, 33 1.00; 32: 2.3 0.95, 33 1.01; 64: 5.5 0.89,
+//     33 1.00, so never
+//   e4m3 keys, D = 128: 16: 0.6 1.05, 2.3 0.96, 9.4 1.16, 33 1.09, so always; 32: 1.9 0.95, 3.2 1.01,
+//     33 1.11; 64: 5.5 0.93, 19 1.01, 33 1.02 / 7.9 0.84, 23 1.02
+//   e4m3 keys, D = 64: 16: 2.3 0.91, 5.5 1.04, 33 1.40 / 6.1 0.94, 7.9 1.14; 32: 5.5 0.95, 11 1.03,
+//     33 1.26; 64: 19 0.97, 29 1.07 / 23 0.99
+//   e4m3 keys and values, D = 128: 16: 0.6 0.95, 3.2 1.10, 33 1.40 / 6.1 0.97, 7.9 1.13; 32: 4.3 0.87,
+//     5.5 1.01, 33 1.30 / 7.9 1.04; 64: 5.5 0.93, 11 1.00, 33 1.22 / 14 1.03
+//   the same at D = 64: 16: 2.3 0.96, 5.5 1.08, 33 1.33 / 7.9 1.17; 32: 7.1 0.87, 12 0.98, 33 1.12 /
+//     18 1.07; 64: 19 0.97, 33 1.04 / 23 1.00
 bool attn_short_ranges(int device, int batch, int kv_heads, int capacity, int head_dim,
                        int rows_max, bool keys_e4m3, bool values_e4m3) {
     const long long pairs = (long long)batch * kv_heads, C = attn_grid_size(device);
-    const long long tiles = pairs * ((capacity + kTileKeys - 1) / kTileKeys + 1);
-    const bool wide = rows_max > 16;
+    const bool many = pairs > C;
+    const int cols = rows_max <= 16 ? 0 : rows_max <= 32 ? 1 : 2;
     int need;
-    if (!keys_e4m3 && !values_e4m3)
-        need = wide ? 9 : 3;
-    else if (!values_e4m3 && head_dim == 128)
-        need = wide ? 9 : 1;
-    else if (head_dim == 128)
-        need = wide ? 11 : pairs > C ? 12 : 4;
-    else
-        need = wide ? 16 : pairs > C ? 12 : 9;
+    if (!keys_e4m3 && !values_e4m3) {
+        if (head_dim == 128) return true;
+        need = cols == 0 ? 10 : cols == 1 ? 22 : 36;
+    } else if (head_dim == 128 && !values_e4m3) {
+        need = cols == 0 ? 0 : cols == 1 ? 6 : many ? 46 : 40;
+    } else if (head_dim == 128) {
+        need = cols == 0 ? (many ? 14 : 8) : cols == 1 ? (many ? 16 : 12) : (many ? 26 : 22);
+    } else if (!values_e4m3) {
+        need = cols == 0 ? (many ? 16 : 12) : cols == 1 ? 22 : many ? 48 : 40;
+    } else {
+        need = cols == 0 ? (many ? 16 : 12) : cols == 1 ? 30 : many ? 46 : 40;
+    }
+    const long long tiles = pairs * (((long long)capacity + kTileKeys - 1) / kTileKeys + 1);
     return tiles < need * (pairs + C);
 }
 

@@ -1,5 +1,6 @@
 """Attention calls on inputs made on the device, and their fp64 reference in plain
 torch: for prefixes too long for the host generator and the oracle."""
+import copy
 import math
 
 import torch
@@ -52,6 +53,28 @@ class Call:
             self.ws = das.new_workspace(self.cache, H * G, rows)
         self.pl = torch.tensor(self.P, dtype=torch.int32, device="cuda")
         self.bl = torch.tensor(self.T, dtype=torch.int32, device="cuda")
+
+    def with_capacity(self, cap):
+        """The same call over a cache of that capacity."""
+        import paper_2609_34538_gb300 as das
+        c = copy.copy(self)
+        k = self.cache.k_top[0] if self.f8 else self.cache.k[1, 0]
+        grown = torch.full((len(self.P), cap) + k.shape[2:], math.nan, dtype=torch.bfloat16,
+                           device="cuda")
+        n = min(cap, k.shape[1])
+        def fit(x):  # [..][B][capacity][H][D]
+            y = grown if x.dtype == torch.bfloat16 else torch.full_like(grown, 0x7F, dtype=torch.uint8)
+            y = y.expand(x.shape[:-4] + y.shape).clone()
+            y[..., :n, :, :] = x[..., :n, :, :]
+            return y
+        if self.f8:
+            c.cache = das.DepthKVCacheF8(*map(fit, (self.cache.k_top, self.cache.v_top,
+                                                    self.cache.k_low, self.cache.v_low)))
+            c.ws = das.new_workspace_f8(c.cache, self.H * self.G, self.q.shape[1])
+        else:
+            c.cache = das.DepthKVCache(fit(self.cache.k), fit(self.cache.v))
+            c.ws = das.new_workspace(c.cache, self.H * self.G, self.q.shape[1])
+        return c
 
     # the stored keys and values that the call reads, [B][cap][H][D] (views, to be edited)
     @property

@@ -1,5 +1,5 @@
 """e4m3 keys scored against queries split into 8-bit parts: rows whose elements span
-many powers of two, over prefixes long enough for the kernel that splits into three
+many powers of two, in caches long enough for the kernel that splits into three
 parts (it has to lose nothing against keys widened to bf16)."""
 import pytest
 import torch
@@ -17,7 +17,7 @@ FORMS = [(64, False), (64, True), (128, True)]  # (D, e4m3 values): three parts
 def test_small_elements_decide(D, vf8, down, G, T):
     """The large elements meet zeros of the keys, so that the scores are those of
     elements 2^-down of the row's largest, times a scale that makes them about 1."""
-    c = Call([9000, 9001, 8963], [T, T, T - 1], G, 8, D, True, vf8, seed=down)
+    c = Call([9000, 9001, 8963], [T, T, T - 1], G, 8, D, True, vf8, 30000, seed=down)
     even = torch.zeros((), device="cuda").to(c.k.dtype)
     c.k[..., ::2] = even
     c.kb[..., ::2] = 0.0
@@ -34,7 +34,7 @@ def test_magnitudes(D, vf8):
     of zeros and one of each extreme bf16 exponent (2^-126 and 2^100, with keys that
     meet zeros)."""
     T = 12
-    c = Call([9000, 9001, 8963], [T] * 3, 4, 8, D, True, vf8, seed=7)
+    c = Call([9000, 9001, 8963], [T] * 3, 4, 8, D, True, vf8, 30000, seed=7)
     for i in range(T):
         c.q[:, i] *= 2.0 ** (i - 8)
         if i % 3 == 0:
