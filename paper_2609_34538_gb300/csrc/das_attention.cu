@@ -521,13 +521,6 @@ __device__ __forceinline__ void lane_reduce(const float (&x)[NC], uint32_t pbuf,
     }
 }
 
-// 1 / x to within an ulp (x > 0; 0 for x = 0)
-__device__ __forceinline__ float inverse(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return x > 0.f ? fmaf(r, fmaf(-x, r, 1.f), r) : 0.f;
-}
-
 // Registers a thread may use, so that a merge CTA (one warp in each of the SM's
 // four register files of 512 x 32) fits beside the attention CTA: 192 with 7
 // warps (two a file) leave 128, 128 with 11 (three a file) too.  bf16 with N = 64 takes

@@ -246,6 +246,15 @@ __device__ __forceinline__ void tmem_fill8(uint32_t taddr, uint32_t x) {
         : "memory");
 }
 
+// 1 / x to within an ulp of the division for x of 1 to 2^120 (0 for x = 0): one step
+// r + r (1 - x r) of Newton's iteration for 1 / r - x = 0 from the hardware's
+// approximation.  (The weights' sums it is for are 1 or more.  Rounded divisions, 32 in
+// a row at a segment's end, took two e4m3 calls of B8 ragged from 81.5 to 87.7 us.)
+__device__ __forceinline__ float inverse(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return x > 0.f ? fmaf(r, fmaf(-x, r, 1.f), r) : 0.f;
+}
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
