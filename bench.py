@@ -138,11 +138,6 @@ def graph_kernel_nodes(graph):
     return kernels
 
 
-def code_digest(path):
-    """code_text_digest of a source file."""
-    return code_text_digest(open(path, encoding="utf-8").read())
-
-
 def code_text_digest(text):
     """First 16 hex digits of the sha256 of a C/C++/CUDA source with its
     comments, trailing blanks and empty lines removed (string and character
@@ -169,12 +164,20 @@ def code_text_digest(text):
     return hashlib.sha256(code.encode()).hexdigest()[:16]
 
 
+ATTENTION_SOURCES = ("das_rows.cu", "das_attention.cu", "das_tc.h", "das_internal.h")
+
+
+def attention_digest(csrc):
+    """code_text_digest of the sources that the attention kernels are compiled from."""
+    return code_text_digest("\n".join(open(os.path.join(csrc, f), encoding="utf-8").read()
+                                      for f in ATTENTION_SOURCES))
+
+
 def kernel_traffic(workload):
     """dram bytes per attention launch from the committed ncu summary, if the
-    kernel's code has not changed since it was captured; else None."""
-    src = os.path.join(ROOT, "paper_2609_34538_gb300", "csrc", "das_attention.cu")
-    digest = code_digest(src)
-    path = os.path.join(ROOT, "profiles", "attn_kernel_traffic.txt")
+    kernels' code has not changed since it was captured; else None."""
+    digest = attention_digest(os.path.join(ROOT, "paper_2609_34538_gb300", "csrc"))
+    path = os.path.join(ROOT, "profiles", "attention_traffic.txt")
     if not os.path.exists(path):
         return None
     for line in open(path):
