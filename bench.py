@@ -465,7 +465,7 @@ def gpu_arm(args):
         "verify_gbs": round(verify_bytes * K_steps / (sum(verify_ms) / 1e3) / 1e9, 1),
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": traffic,
-                     "kernel": "attn_kernel + merge_kernel (one Mature-V layer call)",
+                     "kernel": "rows_kernel + merge_kernel (one Mature-V layer call)",
                      "peak_source": f"{peak_kind} HBM copy bandwidth"},
         "other_workloads": probes,
         "accept_append": commit,
