@@ -196,8 +196,8 @@ das_status attention_core(const Shape &c, int layer, Operand key, Operand value,
     // bf16: the columns are a dimension of their own, outside the positions, so
     // that one {64, keys, panels, 1, 1} box lands as the swizzled panels
     // [panels][keys][64] that the MMAs read (one copy where there were two or four).
-    // (The kernel for short ranges reads bf16 in {64, 1, keys, 1, 1} boxes of the
-    // e4m3 order.)
+    // (das_rows.cu's kernel, short_ranges, reads bf16 in {64, 1, keys, 1, 1} boxes of
+    // the e4m3 order.)
     const bool short_ranges = attn_short_ranges(dev, c.batch, c.kv_heads, c.capacity, D,
                                                 G * max_block, key.e4m3, value.e4m3);
     auto operand_map = [&](CUtensorMap *m, const Operand &o, int keys, int panels, bool swizzle8) {

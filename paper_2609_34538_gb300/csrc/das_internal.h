@@ -47,7 +47,7 @@ size_t attn_workspace_bytes(int device, int batch, int kv_heads, int rows_max, i
 void attn_workspace_layout(void *workspace, int batch, int kv_heads, int rows_max, int head_dim,
                            int num_ctas, AttnParams &p);
 
-// Whether a call's ranges are short enough for the kernel of das_rows.cu.
+// Whether a call takes the kernel of das_rows.cu: short ranges, or bf16 and D = 128.
 bool attn_short_ranges(int device, int batch, int kv_heads, int capacity, int head_dim,
                        int rows_max, bool keys_e4m3, bool values_e4m3);
 

@@ -1,7 +1,8 @@
-// das_rows.cu -- the attention kernel for short ranges: query rows in the lanes
-// of the accumulators (M = 64), one 64-key tile at a time.  das_attention.cu
-// describes the work split, the segments and the merge, and has the kernel for
-// longer ranges; attn_launch says where the line lies.  This one starts sooner (a
+// das_rows.cu -- the attention kernel for bf16 keys and values with 128-wide heads, and
+// for short ranges of every form: query rows in the lanes of the accumulators
+// (M = 64), one 64-key tile at a time.  das_attention.cu describes the work split,
+// the segments and the merge, and has the kernel for longer ranges of the other
+// forms; attn_short_ranges says where the line lies.  This one starts sooner (a
 // row's maximum needs no MMA of its own, a segment ends without sums over the
 // keys), which is what counts where a CTA has a few tiles, and costs more per tile.
 //

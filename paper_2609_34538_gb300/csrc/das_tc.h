@@ -16,8 +16,9 @@ constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kConvWarps = 4;        // query split, e4m3 -> f16 (e4m3 variants)
 constexpr int kPrefetchTiles = 2;    // prefix tiles pulled into L2 before the dependency wait
 constexpr int kLongRange = 80;       // ranges longer than this prefetch none (measured, us per
-                                     // two calls, 2 tiles / 1 / none: verify 108 tiles a range -
-                                     // / 172.6 / 171.4; decode 14 tiles 32.0 / - / 32.9)
+                                     // two calls, 2 tiles / 1 / none: verify, 108 tiles a range,
+                                     // - / 169.3 / 169.4, long - / 166.0 / 165.8; decode, 14
+                                     // tiles, 32.0 / - / 32.9)
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
