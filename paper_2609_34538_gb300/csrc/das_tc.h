@@ -387,9 +387,9 @@ __device__ __forceinline__ void walk_next(const AttnParams &p, Walk &w) {
 // 32 KB (D = 128, bf16), 6 for 16 KB.  A range that holds a block tile takes
 // that many tiles fewer while there is at least one CTA per pair; with more
 // pairs than CTAs nearly every range holds one and the weight would only move
-// work around.  Weights 3 / 5 / 7, us per two calls: B4 P32768 D128 bf16 174.2 /
-// 174.7 / 174.8, ragged B8 D64 bf16 55.6 / 53.8 / 52.7, ragged B8 D128 e4m3 keys
-// and values 84.1 / 82.3 / 83.4.
+// work around.  Weights 3 / 5 / 7 in the transposed kernel, us per two calls: ragged
+// B8 D64 bf16 55.6 / 53.8 / 52.7, ragged B8 D128 e4m3 keys and values 84.1 / 82.3 /
+// 83.4.  (das_rows.cu's kernel: 3, whatever the tile.)
 constexpr int kBlockBytes = 3 * 32768;
 constexpr int kCtasPerPairForWeight = 1;
 

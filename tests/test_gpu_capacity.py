@@ -100,3 +100,15 @@ def test_calls_over_a_long_cache(kf8, vf8, D):
     torch.cuda.synchronize()
     assert c.status() == 2
     assert torch.equal(out, want[3][0]) and torch.equal(lse, want[3][1])
+
+
+@pytest.mark.parametrize("vf8", [False, True])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("cap", [1, 8, 63, 64, 65, 127, 128, 129])
+def test_smallest_caches_of_e4m3_keys(vf8, D, cap):
+    """Up to 16 rows over e4m3 keys with D = 128 always take the kernel that loads two
+    tiles of keys at once: caches of less than that."""
+    c = Call([cap, cap - 1, 0], [3, 1, 2], 2, 4, D, True, vf8, capacity=cap, seed=19)
+    out, lse = c.run()
+    assert_rows(out, lse, c.reference())
+    assert c.status() == 0
