@@ -1809,6 +1809,7 @@ int attn_grid_size(int device) {
 //     5.5 1.01, 33 1.30 / 7.9 1.04; 64: 5.5 0.93, 11 1.00, 33 1.22 / 14 1.03
 //   the same at D = 64: 16: 2.3 0.96, 5.5 1.08, 33 1.33 / 7.9 1.17; 32: 7.1 0.87, 12 0.98, 33 1.12 /
 //     18 1.07; 64: 19 0.97, 33 1.04 / 23 1.00
+// (e4m3 values alone take the lines of e4m3 keys and values.)
 bool attn_short_ranges(int device, int batch, int kv_heads, int capacity, int head_dim,
                        int rows_max, bool keys_e4m3, bool values_e4m3) {
     const long long pairs = (long long)batch * kv_heads, C = attn_grid_size(device);
